@@ -82,6 +82,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar,
   return mbar_wait_bounded_s(smem_addr(bar), parity, limit_ns);
 }
 
+// As mbar_wait_bounded_s, for waits that the threads of a CTA take one by one
+// and agree on later: a thread that gives up sets *failed (shared memory), and
+// threads that still poll give up as soon as they see it.
+__device__ __forceinline__ void mbar_wait_or_flag(uint32_t bar, uint32_t parity,
+                                                  uint64_t limit_ns, volatile int *failed) {
+  if (mbar_try_wait_s(bar, parity)) return;
+  const uint64_t t0 = global_timer_ns();
+  for (uint32_t i = 1; i < (1u << 28); ++i) {
+    if (mbar_try_wait_s(bar, parity)) return;
+    if ((i & 1023u) == 0 && (*failed || global_timer_ns() - t0 > limit_ns)) break;
+  }
+  *failed = 1;
+}
+
 // 3D tiled TMA load of one box into shared memory; completion is signalled
 // on the barrier as transaction bytes. Coordinates are element indices
 // (x innermost) and may lie outside the tensor: those elements read as zero.

@@ -216,7 +216,7 @@ struct SweepCfg {
   static constexpr int THREADS = NTX * NTY;
   static constexpr int SU = PF + 5;           // u ring: 5 live planes + prefetch
   static constexpr int SP = PF + 1;           // u_prev / c ring
-  static constexpr int NB = PF + 1;           // one barrier per in-flight stage
+  static constexpr int NB = SU;               // one barrier per u slot
   static constexpr int UW = TX + 2 * HX;      // u slot row length (elements)
   static constexpr int UH = TY + 2 * kR;
   static constexpr int BOX_U = UW;            // TMA box widths: u with halo,
@@ -230,7 +230,7 @@ struct SweepCfg {
   // 228 KiB / 4 minus the 1 KiB the hardware reserves per CTA.
   static constexpr size_t SMEM_BYTES = (size_t)SU * U_BYTES +
                                        (size_t)SP * (UP_BYTES + C_BYTES) +
-                                       C_BYTES + NB * 8;
+                                       C_BYTES + NB * 8 + 8;
   static_assert(TX % 4 == 0 && TY % VY == 0, "tile shape");
   static_assert((UW * sizeof(T)) % 16 == 0, "TMA box row: multiple of 16 B");
   static_assert((TX * sizeof(T)) % 16 == 0, "TMA box row: multiple of 16 B");
@@ -249,10 +249,10 @@ struct SweepCfg {
 // (112, 176 or 304 bytes: the 8 rows of an ldmatrix land on 8 disjoint
 // groups of 4 banks), u_prev and v^2 dt^2 rows of TX + 8 (the extra columns
 // are the next tile's, read from L2).
-// RING_ = 9: the u_prev / v^2 dt^2 ring and the barriers are 9 deep like
-// the u ring (the plane loop's unroll), so every slot and barrier parity of
-// the loop is a compile-time constant instead of a division by PF + 1 per
-// plane; it needs the shared memory of 2 CTAs per SM or fewer.
+// RING_ = 9: the u_prev / v^2 dt^2 ring is 9 deep like the u ring and the
+// barriers (the plane loop's unroll), so every slot of the loop is a
+// compile-time constant instead of a division by PF + 1 per plane; it needs
+// the shared memory of 2 CTAs per SM or fewer.
 template <int TX_, int PF_, int MINB_, class T_, int RING_ = 0>
 struct TcCfg {
   using T = T_;
@@ -266,7 +266,7 @@ struct TcCfg {
   static constexpr int THREADS = 4 * TX;      // one warp per 8 columns
   static constexpr int SU = PF + 5;
   static constexpr int SP = RING_ ? RING_ : PF + 1;
-  static constexpr int NB = RING_ ? RING_ : PF + 1;
+  static constexpr int NB = SU;
   static constexpr int UW = TX + 24;      // u slot row (elements): x0-8 .. x0+TX+15
   static constexpr int UH = TY + 2 * kR;
   static constexpr int PW = TX + 8;       // u_prev / v^2 dt^2 slot row
@@ -279,7 +279,7 @@ struct TcCfg {
   // rings, then one barrier per stage in flight (receivers are recorded
   // by the threads that own the points: no staging plane)
   static constexpr size_t SMEM_BYTES = (size_t)SU * U_BYTES +
-                                       (size_t)SP * (UP_BYTES + C_BYTES) + NB * 8;
+                                       (size_t)SP * (UP_BYTES + C_BYTES) + NB * 8 + 8;
   static_assert(SU == 9, "the plane loop keeps ring slot = plane mod 9");
   static_assert(U_BYTES % 128 == 0 && UP_BYTES % 128 == 0 && C_BYTES % 128 == 0,
                 "slot alignment");
@@ -297,6 +297,18 @@ __device__ __forceinline__ void acc_exact(float &hi, float &lo, float u, float d
   const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(p, bp));
   hi = s;
   lo = __fadd_rn(lo, __fadd_rn(err, e));
+}
+
+// First entry of e[lo, hi), sorted by depth .x, at depth zb or deeper. A
+// binary search: a walk from lo costs a dependent load per entry (32 a tile
+// with receivers every 4th point), in every CTA below the receiver plane.
+__device__ __forceinline__ int first_at_depth(const int4 *e, int lo, int hi, int zb) {
+  if (zb == 0) return lo;
+  while (lo < hi) {
+    const int mid = lo + ((hi - lo) >> 1);
+    if (e[mid].x < zb) lo = mid + 1; else hi = mid;
+  }
+  return lo;
 }
 
 __device__ __forceinline__ float exp2_int(int k) {
@@ -330,6 +342,8 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
                                         C::SP * C::UP_BYTES);
   float *sr = sc + C::SP * C::P_SLOT;  // receiver staging (one plane)
   uint64_t *bars = reinterpret_cast<uint64_t *>(sr + C::P_SLOT);
+  volatile int *failed = reinterpret_cast<volatile int *>(bars + C::NB);
+  const uint32_t bars_s = smem_addr(bars);
 
   const int tid = threadIdx.x;
   const int tx = tid % C::NTX;
@@ -339,6 +353,40 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
   const int zb = a.zl[bz];
   const int ze = a.zl[bz + 1];
   const int NS = (ze - zb) + 2 * kR;  // stages: 8 to fill the queue, then one per plane
+
+  // Stage s brings u plane zb-4+s and, once s >= 8, u_prev and c of plane
+  // zb-8+s (the plane computed at iteration s).
+  auto issue = [&](int s) {
+    uint64_t *bar = &bars[s % C::NB];
+    const int j = zb - 2 * kR + s;
+    const bool full = j >= zb;
+    mbar_arrive_expect_tx(bar,
+                          C::U_BYTES + (full ? C::UP_BYTES + C::C_BYTES : 0));
+    tma_load_3d(su + (s % C::SU) * C::U_SLOT, tm_u, bar, x0 - C::HX, y0 - kR,
+                j + kR);
+    if (full) {
+      tma_load_3d(sp + (s % C::SP) * C::P_SLOT, tm_up, bar, x0, y0, j);
+      tma_load_3d(sc + (s % C::SP) * C::P_SLOT, tm_c, bar, x0, y0, j);
+    }
+  };
+  // The u ring is empty, so all of its SU stages are issued at once, before
+  // anything else is read: the queue's 8 u-only stages then arrive in about
+  // one load latency instead of two prefetch windows, and the reads of the
+  // per-call state overlap them. A CTA's start and its per-plane latency bound
+  // small grids: with the fill below (1 barrier instead of 8, 0.3 k cycles
+  // instead of 3.3 k) and a plain barrier per plane, a step took 7.9 us
+  // instead of 9.2 at 64^3, 17.1 instead of 18.4 at 203 x 157 x 131, 48.9
+  // instead of 50.6 at 256^3; 1.310 ms instead of 1.327 at 1024 x 1024 x 512,
+  // and 0.989 instead of 1.009 there with FP16 storage.
+  if (tid == 0) {
+    prefetch_tensormap(tm_u);
+    prefetch_tensormap(tm_up);
+    prefetch_tensormap(tm_c);
+    for (int b = 0; b < C::NB; ++b) mbar_init(&bars[b], 1);
+    fence_barrier_init();
+    *failed = 0;
+    for (int s = 0; s < C::SU && s < NS; ++s) issue(s);
+  }
 
   // Per-call state.
   StepDesc *d = a.desc;
@@ -354,7 +402,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
     const int tile = by * a.ntx + bx;
     rcur = d->rec_start[tile];
     rend = d->rec_start[tile + 1];
-    while (rcur < rend && rec[rcur].x < zb) ++rcur;
+    rcur = first_at_depth(rec, rcur, rend, zb);
   }
   int rz = (rcur < rend) ? rec[rcur].x : 0x7fffffff;  // z of the next receiver
   float *trow = (nrec > 0) ? d->traces + (size_t)n * nrec : nullptr;
@@ -368,7 +416,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       irow = d->inj_val + (size_t)n * d->ninj;
       icur = d->inj_start[tile];
       iend = d->inj_start[tile + 1];
-      while (icur < iend && inj[icur].x < zb) ++icur;
+      icur = first_at_depth(inj, icur, iend, zb);
       if (icur < iend) iz = inj[icur].x;
     }
   }
@@ -404,32 +452,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
   }
   float vmax_out = 0.f;  // largest |output| of this thread (stored units)
 
-  if (tid == 0) {
-    prefetch_tensormap(tm_u);
-    prefetch_tensormap(tm_up);
-    prefetch_tensormap(tm_c);
-    for (int b = 0; b < C::NB; ++b) mbar_init(&bars[b], 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-
-  // Stage s brings u plane zb-4+s and, once s >= 8, u_prev and c of plane
-  // zb-8+s (the plane computed at iteration s).
-  auto issue = [&](int s) {
-    uint64_t *bar = &bars[s % C::NB];
-    const int j = zb - 2 * kR + s;
-    const bool full = j >= zb;
-    mbar_arrive_expect_tx(bar,
-                          C::U_BYTES + (full ? C::UP_BYTES + C::C_BYTES : 0));
-    tma_load_3d(su + (s % C::SU) * C::U_SLOT, tm_u, bar, x0 - C::HX, y0 - kR,
-                j + kR);
-    if (full) {
-      tma_load_3d(sp + (s % C::SP) * C::P_SLOT, tm_up, bar, x0, y0, j);
-      tma_load_3d(sc + (s % C::SP) * C::P_SLOT, tm_c, bar, x0, y0, j);
-    }
-  };
-  if (tid == 0)
-    for (int s = 0; s < C::PF && s < NS; ++s) issue(s);
+  __syncthreads();  // the barriers are initialised
 
   // q[v][k]: u of this thread's 4 points on row v. The loop below is unrolled
   // by 9, the queue length, so a plane keeps one register for its whole
@@ -464,19 +487,37 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
   };
   if constexpr ((kMode & kModeGradAcc) != 0) grad_load(zb);
 
+  // The 8 u-only stages fill the queue with one barrier between them: planes
+  // zb-4 .. zb-1 are no one's centre, so once every thread has read them their
+  // slots take the next stages.
   int s = 0;
-  for (int s0 = 0; s0 < NS; s0 += 9) {
 #pragma unroll
-    for (int p = 0; p < 9; ++p) {
-      s = s0 + p;
+  for (int p = 0; p < 2 * kR; ++p) {
+    mbar_wait_or_flag(bars_s + 8u * p, 0, kWaitLimitNs, failed);
+#pragma unroll
+    for (int v = 0; v < C::VY; ++v)
+      q[v][p] = E::load4(su + p * C::U_SLOT + (ty * C::VY + v + kR) * C::UW + col);
+    if (p == kR - 1) {
+      __syncthreads();
+      if (*failed) goto wait_failed;
+      if (tid == 0)
+        for (int t = C::SU; t < 2 * kR + C::PF && t < NS; ++t) issue(t);
+    }
+  }
+  for (int s0 = 2 * kR; s0 < NS; s0 += 9) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const int p = (i + 8) % 9;  // s mod 9: queue register, and u slot
+      s = s0 + i;
       if (s >= NS) break;
-      // One barrier per plane: it publishes that stage s has landed for
-      // every thread (a uniform verdict, so a timeout leaves the loop
-      // everywhere) and that every thread is done with plane s-1, whose
-      // slots the next issue may overwrite.
-      const bool ok =
-          mbar_wait_bounded(&bars[s % C::NB], (s / C::NB) & 1, kWaitLimitNs);
-      if (__syncthreads_or(!ok)) goto wait_failed;
+      // One barrier per plane: stage s has landed for every thread, and
+      // every thread is done with plane s-1, whose slots the next issue may
+      // overwrite. A wait that gave up is looked for every third plane (a
+      // plain barrier is cheaper than one that carries a verdict), before
+      // the failed stage's slot could be issued again.
+      mbar_wait_or_flag(bars_s + 8u * (s % C::NB), (s / C::NB) & 1, kWaitLimitNs, failed);
+      __syncthreads();
+      if (i % 3 == 0 && *failed) goto wait_failed;
       if (tid == 0 && s + C::PF < NS) issue(s + C::PF);
       // Front plane (j+4) into the queue.
       const int fslot = (C::SU == 9) ? p : (s % C::SU);
@@ -485,7 +526,6 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       for (int v = 0; v < C::VY; ++v)
         q[v][p] = E::load4(uf + (ty * C::VY + v + kR) * C::UW + col);
       const int j = zb - 2 * kR + s;
-      if (j < zb) continue;
 
       const int cslot = (C::SU == 9) ? (p + 5) % 9 : ((s + C::SU - kR) % C::SU);
       const T *uc = su + cslot * C::U_SLOT;  // plane j
@@ -722,13 +762,13 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
 
 wait_failed:
   {
-    // A wait gave up at stage s: record it, then drain the stages still in
-    // flight (issued: [0, s + PF)) so no TMA write lands in shared memory
-    // after this CTA has exited.
+    // A wait gave up at stage s or up to four before it: record it, then
+    // drain the stages still in flight (issued: [0, max(SU, s + PF))) so no
+    // TMA write lands in shared memory after this CTA has exited.
     if (tid == 0) {
       atomicCAS(&a.desc->error, 0, kErrTimeout);
-      const int issued = min(NS, s + C::PF);
-      for (int t = s; t < issued; ++t)
+      const int issued = min(NS, max(C::SU, s + C::PF));
+      for (int t = max(0, s - kR); t < issued; ++t)
         if (!mbar_wait_bounded(&bars[t % C::NB], (t / C::NB) & 1, kWaitLimitNs))
           break;
     }
@@ -847,6 +887,7 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
   float *sc = reinterpret_cast<float *>(base + C::SU * C::U_BYTES +
                                         C::SP * C::UP_BYTES);
   uint64_t *bars = reinterpret_cast<uint64_t *>(sc + C::SP * C::P_SLOT);
+  volatile int *failed = reinterpret_cast<volatile int *>(bars + C::NB);
 
   const int tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
@@ -858,6 +899,34 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
   const int zb = a.zl[bz];
   const int ze = a.zl[bz + 1];
   const int NS = (ze - zb) + 2 * kR;
+
+  // Stage t brings u plane zb-4+t (slot t % 9) and, once t >= 8, u_prev and
+  // v^2 dt^2 of plane zb-8+t (the plane computed at iteration t). slot:
+  // t % 9, passed as a constant from the unrolled loop (the ring slots and
+  // barriers are t % 9; the u_prev / v^2 dt^2 ring too when SP == 9).
+  auto issue = [&](int t, int slot9) {
+    const int pslot = C::SP == 9 ? slot9 : t % C::SP;
+    uint64_t *bar = &bars[slot9];
+    const int j = zb - 2 * kR + t;
+    const bool full = j >= zb;
+    mbar_arrive_expect_tx(bar,
+                          C::U_BYTES + (full ? C::UP_BYTES + C::C_BYTES : 0));
+    tma_load_3d(su + slot9 * C::U_SLOT, tm_u, bar, x0 - C::HX, y0 - kR, j + kR);
+    if (full) {
+      tma_load_3d(sp + pslot * C::P_SLOT, tm_up, bar, x0, y0, j);
+      tma_load_3d(sc + pslot * C::P_SLOT, tm_c, bar, x0, y0, j);
+    }
+  };
+  // all 9 slots of the empty u ring at once (see sweep_cta)
+  if (tid == 0) {
+    prefetch_tensormap(tm_u);
+    prefetch_tensormap(tm_up);
+    prefetch_tensormap(tm_c);
+    for (int b = 0; b < C::NB; ++b) mbar_init(&bars[b], 1);
+    fence_barrier_init();
+    *failed = 0;
+    for (int t = 0; t < C::SU && t < NS; ++t) issue(t, t);
+  }
 
   StepDesc *d = a.desc;
   const long long n = d->n + koff;
@@ -873,7 +942,7 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
     const int tile = by * a.ntx + bx;
     rcur = d->rec_start[tile];
     rend = d->rec_start[tile + 1];
-    while (rcur < rend && rec[rcur].x < zb) ++rcur;
+    rcur = first_at_depth(rec, rcur, rend, zb);
   }
   int rz = (rcur < rend) ? rec[rcur].x : 0x7fffffff;
   float *trow = (nrec > 0) ? d->traces + (size_t)n * nrec : nullptr;
@@ -955,56 +1024,43 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
   const bool in_x = x0 + xt < a.px;
   const bool wa = in_x && y0 + g < a.ny, wb = in_x && y0 + g + 8 < a.ny;
 
-  if (tid == 0) {
-    prefetch_tensormap(tm_u);
-    prefetch_tensormap(tm_up);
-    prefetch_tensormap(tm_c);
-    for (int b = 0; b < C::NB; ++b) mbar_init(&bars[b], 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-
-  // Stage t brings u plane zb-4+t (slot t % 9) and, once t >= 8, u_prev and
-  // v^2 dt^2 of plane zb-8+t (the plane computed at iteration t). slot:
-  // t % 9, passed as a constant from the unrolled loop (the ring slots and
-  // barriers are t % 9 when SP == NB == 9).
-  auto issue = [&](int t, int slot9) {
-    const int bslot = C::NB == 9 ? slot9 : t % C::NB;
-    const int pslot = C::SP == 9 ? slot9 : t % C::SP;
-    uint64_t *bar = &bars[bslot];
-    const int j = zb - 2 * kR + t;
-    const bool full = j >= zb;
-    mbar_arrive_expect_tx(bar,
-                          C::U_BYTES + (full ? C::UP_BYTES + C::C_BYTES : 0));
-    tma_load_3d(su + slot9 * C::U_SLOT, tm_u, bar, x0 - C::HX, y0 - kR, j + kR);
-    if (full) {
-      tma_load_3d(sp + pslot * C::P_SLOT, tm_up, bar, x0, y0, j);
-      tma_load_3d(sc + pslot * C::P_SLOT, tm_c, bar, x0, y0, j);
-    }
-  };
-  if (tid == 0)
-    for (int t = 0; t < C::PF && t < NS; ++t) issue(t, t);
+  __syncthreads();  // the barriers are initialised
 
   // q[k]: u of the thread's points (row g: x, y; row g+8: z, w)
   float4 q[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) q[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 
+  // the 8 u-only stages (see sweep_cta)
   int s = 0;
   const int ns_issue = NS - C::PF;  // stages s below it issue stage s + PF
-  uint32_t par9 = 0;  // barrier parity of this round of 9 stages (NB == 9)
-  for (int s0 = 0; s0 < NS; s0 += 9, par9 ^= 1u) {
+  uint32_t par9 = 0;  // barrier parity of the round's first stage
 #pragma unroll
-    for (int p = 0; p < 9; ++p) {
-      s = s0 + p;
+  for (int p = 0; p < 2 * kR; ++p) {
+    mbar_wait_or_flag(bars_s + 8u * p, 0, kWaitLimitNs, failed);
+    const T *uf = su + p * C::U_SLOT;
+    const float2 fa = pair_to_f32<T>(*reinterpret_cast<const unsigned *>(uf + ua));
+    const float2 fb = pair_to_f32<T>(*reinterpret_cast<const unsigned *>(uf + ub));
+    q[p] = make_float4(fa.x, fa.y, fb.x, fb.y);
+    if (p == kR - 1) {
+      __syncthreads();
+      if (*failed) goto wait_failed;
+      if (tid == 0)
+        for (int t = C::SU; t < 2 * kR + C::PF && t < NS; ++t) issue(t, t - C::SU);
+    }
+  }
+  for (int s0 = 2 * kR; s0 < NS; s0 += 9, par9 ^= 1u) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const int p = (i + 8) % 9;  // s mod 9: queue register, slot and barrier
+      s = s0 + i;
       if (s >= NS) break;
-      // One barrier per plane: stage s has landed for every thread (a
-      // uniform verdict, so a timeout leaves the loop everywhere) and every
-      // thread is done with plane s-1, whose slots the next issue reuses.
-      const bool ok =
-          C::NB == 9 ? mbar_wait_bounded_s(bars_s + 8u * p, par9, kWaitLimitNs)
-                     : mbar_wait_bounded(&bars[s % C::NB], (s / C::NB) & 1, kWaitLimitNs);
-      if (__syncthreads_or(!ok)) goto wait_failed;
+      // One barrier per plane: stage s has landed for every thread, and every
+      // thread is done with plane s-1, whose slots the next issue reuses. A
+      // wait that gave up is looked for every third plane (see sweep_cta).
+      mbar_wait_or_flag(bars_s + 8u * p, i == 0 ? par9 : par9 ^ 1u, kWaitLimitNs, failed);
+      __syncthreads();
+      if (i % 3 == 0 && *failed) goto wait_failed;
       if (tid == 0 && s < ns_issue) issue(s + C::PF, (p + C::PF) % 9);
       {
         const T *uf = su + p * C::U_SLOT;  // SU == 9: slot of stage s is s % 9
@@ -1013,9 +1069,7 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
         q[p] = make_float4(fa.x, fa.y, fb.x, fb.y);
       }
       const int j = zb - 2 * kR + s;
-      // j >= zb, i.e. s >= 8: every stage after the first 8 (s0 is a
-      // multiple of 9, so only the first round holds the queue's fill)
-      if (p == 8 || s0 != 0) {
+      {
         const T *uc = su + ((p + 5) % 9) * C::U_SLOT;  // plane j
         const int pslot = C::SP == 9 ? p : s % C::SP;
         const T *pp = sp + pslot * C::P_SLOT;
@@ -1108,13 +1162,13 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
 
 wait_failed:
   {
-    // A wait gave up at stage s: record it, then drain the stages still in
-    // flight (issued: [0, s + PF)) so no TMA write lands in shared memory
-    // after this CTA has exited.
+    // A wait gave up at stage s or up to four before it: record it, then
+    // drain the stages still in flight (issued: [0, max(SU, s + PF))) so no
+    // TMA write lands in shared memory after this CTA has exited.
     if (tid == 0) {
       atomicCAS(&a.desc->error, 0, kErrTimeout);
-      const int issued = min(NS, s + C::PF);
-      for (int t = s; t < issued; ++t)
+      const int issued = min(NS, max(C::SU, s + C::PF));
+      for (int t = max(0, s - kR); t < issued; ++t)
         if (!mbar_wait_bounded(&bars[t % C::NB], (t / C::NB) & 1, kWaitLimitNs))
           break;
     }
