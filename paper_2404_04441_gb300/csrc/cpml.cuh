@@ -14,12 +14,14 @@
 //     C * sum_a ( D1_a psi_a^n + zeta_a^n ),
 // and the axis-a term is non-zero only within w = npml + 4 cells of the two
 // faces normal to a. So the sweep runs unchanged over the whole grid, and
-// afterwards one kernel per axis walks every line along that axis through its
-// two end segments of w cells (one segment of the whole line when the two would
-// overlap): it updates psi_a and zeta_a from u^n (which the sweep does not
-// overwrite) and adds the axis term to u^{n+1}. The three axis kernels run
-// one after another, so corner points are updated by each axis in turn with
-// no race. Receivers within w of a face are then re-recorded.
+// afterwards every line along each axis is walked through its two end segments
+// of w cells (one segment of the whole line when the two would overlap), which
+// updates psi_a and zeta_a from u^n (which the sweep does not overwrite) and
+// adds the axis term to u^{n+1}. Corner points are updated by
+// each axis in turn with no race: where every axis holds two disjoint segments
+// of a width they are unrolled for, by one launch over boxes that own their lines whole
+// and a small second one (cpml_lines_kernel); otherwise by axis passes one
+// after another. Receivers within w of a face are then re-recorded.
 #pragma once
 
 #include <algorithm>
@@ -79,14 +81,23 @@ inline void cpml_axis_coefs(CpmlGeom &g, int ax, double h) {
   }
 }
 
-// Whether an axis of n cells takes the unrolled segment kernels: a layer of
-// 8 or 16 cells, two disjoint end segments (n >= 2 (npml + 4)), and 32-bit
-// per-position offsets (fstep, sstep: the axis's field and slab steps);
+// Widest layer of the unrolled line ends, and the widths they are built for
+// (each unrolls 6 segments); other layers take the line walks.
+constexpr int kCpmlMaxCap = 20;
+constexpr int kCpmlVariants = 4;
+
+inline int cpml_variant(int npml) {
+  return npml == 8 ? 0 : npml == 10 ? 1 : npml == 16 ? 2 : npml == 20 ? 3 : -1;
+}
+
+// Whether an axis of n cells takes the unrolled line ends: a layer width they
+// are built for, two disjoint end segments (n >= 2 (npml + 4)), and 32-bit
+// offsets along the line (fstep, sstep: the axis's field and slab steps);
 // GBWAVE_CPML_GENERIC=1 keeps the line walks everywhere (the two forms give
 // bitwise equal results).
 inline bool cpml_seg_fits(int npml, int n, long long fstep, long long sstep) {
   const char *gen = std::getenv("GBWAVE_CPML_GENERIC");
-  return (npml == 8 || npml == 16) && n >= 2 * (npml + 4) &&
+  return cpml_variant(npml) >= 0 && n >= 2 * (npml + 4) &&
          (long long)(npml + 3) * fstep <= INT32_MAX &&
          (long long)(npml - 1) * sstep <= INT32_MAX && !(gen && std::atoi(gen) == 1);
 }
@@ -500,126 +511,270 @@ __global__ void __launch_bounds__(128)
   }
 }
 
-// Unrolled segment kernels for layers of NPML = 8 or 16 cells, on axes
-// where the two end segments are disjoint (n >= 2 w): one thread per line
-// end (blockIdx.z: 0 the low face, 1 the high face), so the two segments of
-// a line run in parallel. Positions are counted from the face, j = 0 .. w-1
-// (i = j, or i = n-1-j at the high face); mirroring flips the sign of D1,
-// which the kernels fold into the order of each difference, so every
-// operation rounds exactly as in the line walks above (the results are
-// bitwise equal). With NPML fixed the whole segment is unrolled: u^n is read
-// at the w positions the layer needs (psi reaches u up to npml + 3 cells from
-// the face), psi and zeta at the npml slab cells, C and u^{n+1} at the w
-// correction points, with no per-position predicates; the profile values
-// travel in the kernel's parameters (constant operands of the FMAs).
+// ---------------------------------------------------------------------------
+// The layer in one launch.
+//
+// The three axis terms of a step meet only where shells cross: the axis-a
+// term of a point needs u^n, psi_a and zeta_a along its own line, inside one
+// end segment of w = npml + 4 cells, and nothing else. So the shell splits
+// into boxes by whether each coordinate lies near a low face, between, or
+// near a high one, and every box owns its lines whole:
+//   * faces (one coordinate near a face): the lines normal to it;
+//   * edges (two, tiled by T cells along the third axis): the lines of the
+//     lower axis, then, after a barrier, those of the higher one, which add to
+//     the points the first ones wrote;
+//   * corners: x, then y, then z lines.
+// Every point gets its x, y and z terms in that order, as three axis passes
+// one after another would add them: the results are bitwise the same. A box's
+// lines are shared by a cluster of kCpmlCluster CTAs, so that an edge tile is
+// wide enough for whole sectors along x and still takes one line per thread
+// and phase; the barrier is the cluster's.
+//
+// A line end is one thread: positions are counted from the face (j = 0 ..
+// w-1, mirrored at the high face, where D1 changes sign: folded into the order
+// of each difference, so every operation rounds as in the line walks above).
+// The segment of a layer of NPML cells is unrolled with no per-position
+// predicates: u^n is read only at the w positions the layer needs (psi reaches
+// u up to npml + 3 cells from the face), the profile values travel in the
+// kernel's parameters (constant operands), offsets along the line are 32-bit.
+//
+// What bounds it: on small grids the launches and two memory latencies a
+// line (u^n, psi and zeta; then C and u^{n+1}), on large ones the traffic of
+// lines that every array is read along. Against one launch per axis (line
+// walks at 10 cells, unrolled at 16), a whole step took 31 us instead of 56
+// at 150 x 141 x 133 with 10 cells, 102 instead of 104 at 320 x 256 x 192 in
+// FP16 and 291 instead of 296 at 512 x 512 x 256 with 16; the gradient through
+// autograd at 160 x 144 x 128 x 100 steps 18.0 ms instead of 20.0. CTAs of 256
+// threads without clusters took 7 % longer at 320 x 256 x 192, 4 CTAs an SM
+// (128 registers) 2 %, a second launch for the corners' z lines instead of the
+// third phase 4 %, L2 prefetches of C and u^{n+1} 10 %.
+constexpr int kCpmlThreads = 128;
+constexpr int kCpmlCluster = 4;
+constexpr int kCpmlLines = kCpmlThreads * kCpmlCluster;  // lines of a cluster
+
+// CTAs per SM the line kernels are compiled for (168 registers a thread up to 16 cells, 255 beyond).
+constexpr int cpml_ctas(int npml) { return npml > 16 ? 2 : 3; }
+
+// Profile values by axis, face and depth from the face.
 template <int NPML>
-struct CpmlSideProf {
-  float b[2][NPML], a[2][NPML];  // [face][j], j counted from the face
+struct CpmlProf {
+  float b[3][2][NPML], a[3][2][NPML];
 };
 
-// Profile values of an axis of n cells (b, a along the axis) by face and
-// depth from the face.
 template <int NPML>
-inline void cpml_side_prof(const float *b, const float *a, int n, CpmlSideProf<NPML> &pf) {
-  for (int j = 0; j < NPML; ++j)
+inline void cpml_fill_prof(CpmlProf<NPML> &pf, int ax, const float *b, const float *a, int n,
+                           int npml) {
+  for (int j = 0; j < NPML && j < npml; ++j)
     for (int sd = 0; sd < 2; ++sd) {
       const int i = sd ? n - 1 - j : j;
-      pf.b[sd][j] = b[i];
-      pf.a[sd][j] = a[i];
+      pf.b[ax][sd][j] = b[i];
+      pf.a[ax][sd][j] = a[i];
     }
 }
 
-// Segment addressing shared by the unrolled kernels: line offset of
-// position j (field layout) and of slab cell j (slab layout).
-// The per-position steps are 32-bit (the host takes these kernels only
-// where (w - 1) times the field step and (npml - 1) times the slab step fit
-// in an int), which keeps one register per offset instead of a 64-bit
-// address for each of the segment's loads and stores.
-struct CpmlSeg {
-  long long u0;  // field offset of j = 0 (pitch pxu)
-  long long c0;  // v^2 dt^2 offset of j = 0 (pitch px)
-  long long s0;  // slab offset of j = 0
-  int ustep;     // per-position field step
-  int cstep;     // per-position v^2 dt^2 step
-  int sstep;     // per-cell slab step
-  int n;
+// Clusters of one launch: the corners, the edges of each pair of axes, then
+// the faces of each axis. all: every axis at once; otherwise the lines of one
+// axis alone, over the whole grid (a layer with an axis too short for two
+// disjoint segments takes its axes one by one).
+struct CpmlTiles {
+  int w, T;
+  int near[3];   // cells near a face: w, along x rounded up to 8 (whole
+                 // sectors for the y and z faces) where the grid allows
+  int all;
+  int start[8];  // corners; xy, xz, yz edges; x, y, z faces; total
+  struct {
+    int half;               // clusters of one side
+    int p0, np, q0, total;  // cross coordinates and lines of a side
+  } face[3];
 };
 
-// t: index across the lines, q: row of lines (z for x and y lines, y for
-// z lines).
-template <int AX, int NPML>
-__device__ __forceinline__ bool cpml_seg_setup(const CpmlGeom &g, int side, int t, int q,
-                                               CpmlSeg &sg) {
-  long long ub, us, cb, cs, sb, ss;
-  if (AX == 0) {
-    if (t >= g.ny) return false;
-    sg.n = g.nx;
-    ub = ((long long)q * g.ny + t) * g.pxu;
-    us = 1;
-    cb = ((long long)q * g.ny + t) * g.px;
-    cs = 1;
-    sb = (long long)q * g.ny + t;
-    ss = (long long)g.nz * g.ny;
-  } else {
-    if (t >= g.nx) return false;
-    sg.n = AX == 1 ? g.ny : g.nz;
-    ub = AX == 1 ? (long long)q * g.ny * g.pxu + t : (long long)q * g.pxu + t;
-    us = AX == 1 ? (long long)g.pxu : (long long)g.ny * g.pxu;
-    cb = AX == 1 ? (long long)q * g.ny * g.px + t : (long long)q * g.px + t;
-    cs = AX == 1 ? (long long)g.px : (long long)g.ny * g.px;
-    sb = (long long)q * g.nx + t;
-    ss = AX == 1 ? (long long)g.nz * g.nx : (long long)g.ny * g.nx;
+inline CpmlTiles cpml_tiles(int nx, int ny, int nz, int w, int only) {
+  CpmlTiles t{};
+  t.w = w;
+  t.all = only < 0;
+  const int n[3] = {nx, ny, nz};
+  long long nb[7] = {};
+  if (t.all) {
+    const int r8 = (w + 7) & ~7;
+    t.near[0] = 2 * r8 <= nx ? r8 : w;
+    t.near[1] = t.near[2] = w;
+    t.T = std::max(4, (kCpmlLines / t.near[0]) & ~3);
+    nb[0] = 8;
+    for (int e = 0; e < 3; ++e)
+      nb[1 + e] = 4ll * ((n[2 - e] - 2 * t.near[2 - e] + t.T - 1) / t.T);
   }
-  // the high face's slab cell of position j is 2 npml - 1 - j
-  sg.u0 = side ? ub + (long long)(sg.n - 1) * us : ub;
-  sg.ustep = (int)(side ? -us : us);
-  sg.c0 = side ? cb + (long long)(sg.n - 1) * cs : cb;
-  sg.cstep = (int)(side ? -cs : cs);
-  sg.s0 = side ? sb + (long long)(2 * NPML - 1) * ss : sb;
-  sg.sstep = (int)(side ? -ss : ss);
-  return true;
+  for (int ax = 0; ax < 3; ++ax) {
+    if (!t.all && ax != only) continue;
+    const int b = ax == 0 ? 1 : 0, c = ax == 2 ? 1 : 2;
+    const long long p = n[b] - 2 * t.near[b], q = n[c] - 2 * t.near[c];
+    t.face[ax].half = (int)((p * q + kCpmlLines - 1) / kCpmlLines);
+    t.face[ax].p0 = t.near[b];
+    t.face[ax].np = (int)p;
+    t.face[ax].q0 = t.near[c];
+    t.face[ax].total = (int)(p * q);
+    nb[4 + ax] = 2ll * t.face[ax].half;
+  }
+  for (int k = 0; k < 7; ++k) t.start[k + 1] = t.start[k] + (int)nb[k];
+  return t;
 }
 
-// W = NPML + 4 values of a field along the segment, v[j] = f(position j)
-// (base: offset of j = 0, step: per position), times s (16-bit fields).
-// x lines are rows: read as 4-element vectors when the segment starts on a
-// vector boundary (the low face always; the high face when n is a multiple
+__host__ __device__ __forceinline__ int cpml_dim(const CpmlGeom &g, int ax) {
+  return ax == 0 ? g.nx : ax == 1 ? g.ny : g.nz;
+}
+
+// A rectangle of lines: axis ax, face side, cross coordinates p in [p0, p0 +
+// np) and q in [q0, q0 + nq), p along the lower of the two other axes (adjacent
+// lines in adjacent threads).
+struct CpmlRect {
+  int ax, side, p0, np, q0, nq;
+};
+
+// A range of cells along one axis.
+struct CpmlRange {
+  int lo, n;
+};
+
+// The lines of cluster blk, in its phases. ctid: thread within the cluster;
+// line(ax, side, p, q) takes a line, sync() is the cluster's barrier.
+#pragma nv_exec_check_disable
+template <class F, class S>
+__host__ __device__ __forceinline__ void cpml_block(const CpmlGeom &g, const CpmlTiles &t,
+                                                    int blk, int ctid, const F &line,
+                                                    const S &sync) {
+  CpmlRange r[3];
+  unsigned sides, axes;
+  int phases, ax = -1;
+  CpmlRange p, q;
+  int total, first = ctid, step = kCpmlLines;
+  const bool face = blk >= t.start[4];
+  if (face) {  // most blocks: one line a thread
+    ax = blk >= t.start[6] ? 2 : blk >= t.start[5] ? 1 : 0;
+    const auto &f = ax == 2 ? t.face[2] : ax == 1 ? t.face[1] : t.face[0];
+    const int local = blk - (ax == 2 ? t.start[6] : ax == 1 ? t.start[5] : t.start[4]);
+    const int side = local >= f.half;
+    first += (local - (side ? f.half : 0)) * kCpmlLines;
+    total = f.total;
+    step = 1 << 30;
+    p = CpmlRange{f.p0, f.np};
+    q = CpmlRange{f.q0, 0};
+    sides = side ? 7u : 0u;
+    axes = 0;
+    phases = 1;
+  } else {
+    auto near_range = [&](int k, int side) {
+      return CpmlRange{side ? cpml_dim(g, k) - t.near[k] : 0, t.near[k]};
+    };
+    if (blk < 8) {  // corners
+      axes = 7;
+      sides = (unsigned)blk;
+      phases = 3;
+    } else {  // a tile of an edge along m
+      const int cls = blk >= t.start[3] ? 3 : blk >= t.start[2] ? 2 : 1;
+      const int local = blk - (cls == 3 ? t.start[3] : cls == 2 ? t.start[2] : t.start[1]);
+      const int m = 3 - cls, a = cls == 3 ? 1 : 0, b = cls == 1 ? 1 : 2;
+      const int nr = m == 0 ? t.near[0] : t.w, len = cpml_dim(g, m) - 2 * nr;
+      const int per = (len + t.T - 1) / t.T, ci = local / per, m0 = (local - ci * per) * t.T;
+      axes = (1u << a) | (1u << b);
+      sides = ((ci & 1u) << a) | ((unsigned)(ci >> 1) << b);
+      phases = 2;
+      r[0] = r[1] = r[2] = CpmlRange{nr + m0, len - m0 < t.T ? len - m0 : t.T};
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      if ((axes >> k) & 1) r[k] = near_range(k, (sides >> k) & 1);
+  }
+#pragma unroll 1
+  for (int ph = 0; ph < phases; ++ph) {
+    if (!face) {
+      if (ph) sync();
+      do ++ax;
+      while (!((axes >> ax) & 1));
+      p = ax == 0 ? r[1] : r[0];
+      q = ax == 2 ? r[1] : r[2];
+      total = p.n * q.n;
+    }
+#pragma unroll 1
+    for (int i = first; i < total; i += step) {
+      const int iq = (int)((unsigned)i / (unsigned)p.n);
+      line(ax, (int)((sides >> ax) & 1), p.lo + (i - iq * p.n), q.lo + iq);
+      if (face) break;
+    }
+  }
+}
+
+// Offsets of a line end: field (pitch pxu), v^2 dt^2 (pitch px) and slab of
+// position j = 0, and the steps per position. The high face's slab cell of
+// position j is 2 npml - 1 - j.
+struct CpmlLine {
+  long long u0, c0, s0;
+  int ustep, cstep, sstep, n;
+};
+
+template <int AX, int SIDE>
+__device__ __forceinline__ CpmlLine cpml_line_at(const CpmlGeom &g, int p, int q) {
+  CpmlLine l;
+  l.n = AX == 0 ? g.nx : AX == 1 ? g.ny : g.nz;
+  const int x = AX == 0 ? 0 : p, y = AX == 0 ? p : AX == 1 ? 0 : q, z = AX == 2 ? 0 : q;
+  const int us = AX == 0 ? 1 : AX == 1 ? g.pxu : g.ny * g.pxu;
+  const int cs = AX == 0 ? 1 : AX == 1 ? g.px : g.ny * g.px;
+  // slabs: ((cell nz + z) ny + y), ((cell nz + z) nx + x), ((cell ny + y) nx + x)
+  const int ss = AX == 0 ? g.nz * g.ny : AX == 1 ? g.nz * g.nx : g.ny * g.nx;
+  const long long row = (long long)z * g.ny + y;
+  l.u0 = row * g.pxu + x;
+  l.c0 = row * g.px + x;
+  l.s0 = AX == 0 ? row : AX == 1 ? (long long)z * g.nx + x : (long long)y * g.nx + x;
+  if (SIDE) {
+    l.u0 += (long long)(l.n - 1) * us;
+    l.c0 += (long long)(l.n - 1) * cs;
+    l.s0 += (long long)(2 * g.npml - 1) * ss;
+  }
+  l.ustep = SIDE ? -us : us;
+  l.cstep = SIDE ? -cs : cs;
+  l.sstep = SIDE ? -ss : ss;
+  return l;
+}
+
+// v[j] = f(position j) times s for the W positions (r: position
+// 0). x lines are rows: read as 4-element vectors when the segment starts on
+// a vector boundary (the low face always; the high face when n is a multiple
 // of 4).
-template <int AX, int W, int SIDE, class T>
-__device__ __forceinline__ void cpml_seg_load(const T *f, long long base, int step, int n,
-                                              float s, float *v) {
+template <int AX, int SIDE, int W, class T>
+__device__ __forceinline__ void cpml_line_load(const T *r, int step, int n, float s,
+                                               float *v) {
   if (AX == 0 && (SIDE == 0 || (n & 3) == 0)) {
-    const T *r = SIDE == 0 ? f + base : f + base - (W - 1);
 #pragma unroll
     for (int k = 0; k < W; k += 4) {
       float e[4];
-      cpml_get4(r + k, s, e);
+      cpml_get4(SIDE == 0 ? r + k : r - (k + 3), s, e);
 #pragma unroll
-      for (int m = 0; m < 4; ++m) v[SIDE == 0 ? k + m : W - 1 - (k + m)] = e[m];
+      for (int m = 0; m < 4; ++m)
+        if (k + m < W) v[k + m] = SIDE == 0 ? e[m] : e[3 - m];
     }
   } else {
-    const T *r = f + base;
 #pragma unroll
-    for (int j = 0; j < W; ++j) v[j] = cpml_get(r + j * step, s);
+    for (int j = 0; j < W; ++j)
+      v[j] = cpml_get(r + j * step, s);
   }
 }
 
-template <int AX, int W, int SIDE, class T>
-__device__ __forceinline__ void cpml_seg_store(T *f, long long base, int step, int n,
-                                               float inv, const float *v) {
-  if (AX == 0 && (SIDE == 0 || (n & 3) == 0)) {
-    T *r = SIDE == 0 ? f + base : f + base - (W - 1);
+// A group of 4 that reaches past the segment is stored one by one: the points
+// behind it may belong to another cluster.
+template <int AX, int SIDE, int W, class T>
+__device__ __forceinline__ void cpml_line_store(T *r, int step, int n, float inv,
+                                                const float *v) {
+  const bool vec = AX == 0 && (SIDE == 0 || (n & 3) == 0);
 #pragma unroll
-    for (int k = 0; k < W; k += 4) {
+  for (int k = 0; k < W; k += 4) {
+    if (vec && k + 4 <= W) {
       float e[4];
 #pragma unroll
-      for (int m = 0; m < 4; ++m) e[m] = v[SIDE == 0 ? k + m : W - 1 - (k + m)];
-      cpml_put4(r + k, e, inv);
-    }
-  } else {
-    T *r = f + base;
+      for (int m = 0; m < 4; ++m) e[m] = k + 4 <= W ? v[SIDE == 0 ? k + m : k + 3 - m] : 0.f;
+      cpml_put4(SIDE == 0 ? r + k : r - (k + 3), e, inv);
+    } else {
 #pragma unroll
-    for (int j = 0; j < W; ++j) cpml_put(r + j * step, v[j], inv);
+      for (int m = 0; m < 4; ++m)
+        if (k + m < W) cpml_put(r + (k + m) * step, v[k + m], inv);
+    }
   }
 }
 
@@ -654,37 +809,32 @@ __device__ __forceinline__ float cpml_seg_d2(const float *v, int j, const float 
   return d;
 }
 
-template <int AX, int NPML, class T, bool kStoreD, int SIDE>
-__device__ __forceinline__ void cpml_seg_forward(const CpmlGeom &g, const CpmlSideProf<NPML> &pf,
-                                                 int t, int q, const T *__restrict__ u,
-                                                 T *__restrict__ unext,
-                                                 const float *__restrict__ c,
-                                                 float *__restrict__ dout,
-                                                 const StepDesc *d, int koff) {
+// One line end of the forward step. Two phases, each issuing all of its loads
+// before its first store (the slabs and the fields are not known to be
+// distinct, so a load after a store waits for it): u^n, psi and zeta -> the
+// new psi, zeta and the corrections; then C, u^{n+1} (and D) -> u^{n+1} (and
+// D) updated. The live set stays about half of what one phase would hold.
+// T: the wavefields' storage (float, or 16-bit with the step's scales); D is
+// stored for FP32 only.
+template <int AX, int SIDE, int NPML, class T, bool kStoreD, class P>
+__device__ __forceinline__ void cpml_line_forward(const CpmlGeom &g, const P &pf, int p, int q,
+                                                  const T *u, T *unext, const float *c,
+                                                  float *dout, const CpmlScale<T> &sc) {
   constexpr int W = NPML + 4;
-  CpmlSeg sg;
-  if (!cpml_seg_setup<AX, NPML>(g, SIDE, t, q, sg)) return;
-  CpmlScale<T> sc;
-  sc.init(d, koff);
-  float *psi = g.psi[AX] + sg.s0;
-  float *zeta = g.zeta[AX] + sg.s0;
-  // Two phases, each issuing all of its loads before its first store (the
-  // slabs and the fields are not known to be distinct, so a load after a
-  // store waits for it): u^n, psi and zeta -> the new psi, zeta and the
-  // corrections; then C, u^{n+1} (and D) -> u^{n+1} (and D) updated. The
-  // second phase's loads wait behind the slab stores once per thread, and
-  // the live set stays about half of what one phase would hold.
+  const CpmlLine l = cpml_line_at<AX, SIDE>(g, p, q);
+  float *psi = g.psi[AX] + l.s0;
+  float *zeta = g.zeta[AX] + l.s0;
   float U[W], PS[NPML], ZT[NPML], CORR[W];
-  cpml_seg_load<AX, W, SIDE>(u, sg.u0, sg.ustep, sg.n, sc.su, U);
+  cpml_line_load<AX, SIDE, W>(u + l.u0, l.ustep, l.n, sc.su, U);
 #pragma unroll
   for (int j = 0; j < NPML; ++j) {
-    PS[j] = psi[j * sg.sstep];
-    ZT[j] = zeta[j * sg.sstep];
+    PS[j] = psi[j * l.sstep];
+    ZT[j] = zeta[j * l.sstep];
   }
 #pragma unroll
   for (int j = 0; j < NPML; ++j) {
     const float d1 = cpml_seg_d1<SIDE, W>(U, j, g.c1[AX]);
-    PS[j] = fmaf(pf.b[SIDE][j], PS[j], pf.a[SIDE][j] * d1);
+    PS[j] = fmaf(pf.b[AX][SIDE][j], PS[j], pf.a[AX][SIDE][j] * d1);
   }
 #pragma unroll
   for (int j = 0; j < W; ++j) {
@@ -692,22 +842,23 @@ __device__ __forceinline__ void cpml_seg_forward(const CpmlGeom &g, const CpmlSi
     CORR[j] = d1p;
     if (j < NPML) {
       const float d2 = cpml_seg_d2<W>(U, j, g.c2[AX]);
-      ZT[j] = fmaf(pf.b[SIDE][j], ZT[j], pf.a[SIDE][j] * (d2 + d1p));
+      ZT[j] = fmaf(pf.b[AX][SIDE][j], ZT[j], pf.a[AX][SIDE][j] * (d2 + d1p));
       CORR[j] += ZT[j];
     }
   }
 #pragma unroll
   for (int j = 0; j < NPML; ++j) {
-    psi[j * sg.sstep] = PS[j];
-    zeta[j * sg.sstep] = ZT[j];
+    psi[j * l.sstep] = PS[j];
+    zeta[j * l.sstep] = ZT[j];
   }
   float CC[W], UN[W], DO[kStoreD ? W : 1];
   if constexpr (std::is_same<T, float>::value)  // FP32 storage: pxu == px
-    cpml_seg_load<AX, W, SIDE>(c, sg.u0, sg.ustep, sg.n, 1.f, CC);
+    cpml_line_load<AX, SIDE, W>(c + l.u0, l.ustep, l.n, 1.f, CC);
   else
-    cpml_seg_load<AX, W, SIDE>(c, sg.c0, sg.cstep, sg.n, 1.f, CC);
-  cpml_seg_load<AX, W, SIDE>(unext, sg.u0, sg.ustep, sg.n, sc.so, UN);
-  if constexpr (kStoreD) cpml_seg_load<AX, W, SIDE>(dout, sg.u0, sg.ustep, sg.n, 1.f, DO);
+    cpml_line_load<AX, SIDE, W>(c + l.c0, l.cstep, l.n, 1.f, CC);
+  cpml_line_load<AX, SIDE, W>((const T *)unext + l.u0, l.ustep, l.n, sc.so, UN);
+  if constexpr (kStoreD)
+    cpml_line_load<AX, SIDE, W>((const float *)dout + l.u0, l.ustep, l.n, 1.f, DO);
   float vmax = 0.f;
 #pragma unroll
   for (int j = 0; j < W; ++j) {
@@ -715,96 +866,143 @@ __device__ __forceinline__ void cpml_seg_forward(const CpmlGeom &g, const CpmlSi
     vmax = fmaxf(vmax, fabsf(UN[j]));
     if constexpr (kStoreD) DO[j] = fmaf(CC[j], CORR[j], DO[j]);
   }
-  cpml_seg_store<AX, W, SIDE>(unext, sg.u0, sg.ustep, sg.n, sc.inv_so, UN);
-  if constexpr (kStoreD) cpml_seg_store<AX, W, SIDE>(dout, sg.u0, sg.ustep, sg.n, 1.f, DO);
+  cpml_line_store<AX, SIDE, W>(unext + l.u0, l.ustep, l.n, sc.inv_so, UN);
+  if constexpr (kStoreD)
+    cpml_line_store<AX, SIDE, W>(dout + l.u0, l.ustep, l.n, 1.f, DO);
   sc.commit(vmax);
 }
 
-// T: the wavefields' storage (float, or 16-bit with the step's scales read
-// from d at absolute step step0 + n + koff); D is stored for FP32 only.
-template <int AX, int NPML, class T, bool kStoreD = false>
-__global__ void __launch_bounds__(128)
-    cpml_seg_kernel(CpmlGeom g, CpmlSideProf<NPML> pf, const T *__restrict__ u,
-                    T *__restrict__ unext, const float *__restrict__ c,
-                    float *__restrict__ dout, const StepDesc *d, int koff) {
-  static_assert(!kStoreD || std::is_same<T, float>::value, "D is stored for FP32 only");
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
-  if (blockIdx.z == 0)
-    cpml_seg_forward<AX, NPML, T, kStoreD, 0>(g, pf, t, q, u, unext, c, dout, d, koff);
-  else
-    cpml_seg_forward<AX, NPML, T, kStoreD, 1>(g, pf, t, q, u, unext, c, dout, d, koff);
-}
-
-// The adjoint's segment form (cpml_adjoint_line_kernel, unrolled): nu and
-// g = p^{k+1} + A nu at the w positions, mu at the slab cells, then
-// p^k += C (D2 (A nu) - D1 (A mu)) over the segment.
-template <int AX, int NPML, int SIDE>
-__device__ __forceinline__ void cpml_seg_adjoint(const CpmlGeom &g, const CpmlSideProf<NPML> &pf,
-                                                 const float *__restrict__ p1,
-                                                 float *__restrict__ p0,
-                                                 const float *__restrict__ c,
-                                                 float *__restrict__ nus,
-                                                 float *__restrict__ mus) {
+// One line end of the adjoint step (cpml_adjoint_line_kernel, unrolled): nu
+// and g = p^{k+1} + A nu at the w positions, mu at the slab cells, then p^k +=
+// C (D2 (A nu) - D1 (A mu)) over the segment; two phases as in the forward.
+template <int AX, int SIDE, int NPML, class P>
+__device__ __forceinline__ void cpml_line_adjoint(const CpmlGeom &g, const P &pf, int p, int q,
+                                                  const float *p1, float *p0, const float *c,
+                                                  float *nus, float *mus) {
   constexpr int W = NPML + 4;
-  CpmlSeg sg;
-  if (!cpml_seg_setup<AX, NPML>(g, SIDE, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y,
-                                sg))
-    return;
-  float *nu = nus + sg.s0;
-  float *mu = mus + sg.s0;
-  // two phases as in the forward: p^{k+1}, nu, mu -> nu, mu and the
-  // corrections; then C, p^k -> p^k updated
-  float P[W], G[W], NU[NPML], MU[NPML], AN[NPML], AM[NPML], CORR[W];
-  cpml_seg_load<AX, W, SIDE>(p1, sg.u0, sg.ustep, sg.n, 1.f, P);
+  const CpmlLine l = cpml_line_at<AX, SIDE>(g, p, q);
+  float *nu = nus + l.s0, *mu = mus + l.s0;
+  float G[W], NU[NPML], MU[NPML], AN[NPML], AM[NPML], CORR[W];
+  cpml_line_load<AX, SIDE, W>(p1 + l.u0, l.ustep, l.n, 1.f, G);
 #pragma unroll
   for (int j = 0; j < NPML; ++j) {
-    NU[j] = nu[j * sg.sstep];
-    MU[j] = mu[j * sg.sstep];
-  }
-#pragma unroll
-  for (int j = 0; j < W; ++j) {
-    G[j] = P[j];
-    if (j < NPML) {
-      NU[j] = fmaf(pf.b[SIDE][j], NU[j], P[j]);
-      AN[j] = __fmul_rn(pf.a[SIDE][j], NU[j]);
-      G[j] = __fadd_rn(P[j], AN[j]);  // as the line walk: no contraction
-    }
+    NU[j] = nu[j * l.sstep];
+    MU[j] = mu[j * l.sstep];
   }
 #pragma unroll
   for (int j = 0; j < NPML; ++j) {
-    const float d1 = cpml_seg_d1<SIDE, W>(G, j, g.c1[AX]);
-    MU[j] = fmaf(pf.b[SIDE][j], MU[j], -d1);
-    AM[j] = __fmul_rn(pf.a[SIDE][j], MU[j]);
+    NU[j] = fmaf(pf.b[AX][SIDE][j], NU[j], G[j]);
+    AN[j] = __fmul_rn(pf.a[AX][SIDE][j], NU[j]);
+    G[j] = __fadd_rn(G[j], AN[j]);  // as the line walk: no contraction
   }
 #pragma unroll
-  for (int j = 0; j < W; ++j) {
-    // A nu and A mu are zero past the slab
+  for (int j = 0; j < NPML; ++j) {
+    MU[j] = fmaf(pf.b[AX][SIDE][j], MU[j], -cpml_seg_d1<SIDE, W>(G, j, g.c1[AX]));
+    AM[j] = __fmul_rn(pf.a[AX][SIDE][j], MU[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < W; ++j) {  // A nu and A mu are zero past the slab
     const float d2 = cpml_seg_d2<NPML>(AN, j, g.c2[AX]);
     const float d1 = cpml_seg_d1<SIDE, NPML>(AM, j, g.c1[AX]);
     CORR[j] = d2 - d1;
   }
 #pragma unroll
   for (int j = 0; j < NPML; ++j) {
-    nu[j * sg.sstep] = NU[j];
-    mu[j * sg.sstep] = MU[j];
+    nu[j * l.sstep] = NU[j];
+    mu[j * l.sstep] = MU[j];
   }
   float CC[W], PO[W];
-  cpml_seg_load<AX, W, SIDE>(c, sg.u0, sg.ustep, sg.n, 1.f, CC);  // FP32: pxu == px
-  cpml_seg_load<AX, W, SIDE>(p0, sg.u0, sg.ustep, sg.n, 1.f, PO);
+  cpml_line_load<AX, SIDE, W>(c + l.u0, l.ustep, l.n, 1.f, CC);  // FP32: pxu == px
+  cpml_line_load<AX, SIDE, W>((const float *)p0 + l.u0, l.ustep, l.n, 1.f, PO);
 #pragma unroll
-  for (int j = 0; j < W; ++j) PO[j] = fmaf(CC[j], CORR[j], PO[j]);
-  cpml_seg_store<AX, W, SIDE>(p0, sg.u0, sg.ustep, sg.n, 1.f, PO);
+  for (int j = 0; j < W; ++j)
+    PO[j] = fmaf(CC[j], CORR[j], PO[j]);
+  cpml_line_store<AX, SIDE, W>(p0 + l.u0, l.ustep, l.n, 1.f, PO);
 }
 
-template <int AX, int NPML>
-__global__ void __launch_bounds__(128)
-    cpml_seg_adjoint_kernel(CpmlGeom g, CpmlSideProf<NPML> pf, const float *__restrict__ p1,
-                            float *__restrict__ p0, const float *__restrict__ c,
-                            float *__restrict__ nus, float *__restrict__ mus) {
-  if (blockIdx.z == 0)
-    cpml_seg_adjoint<AX, NPML, 0>(g, pf, p1, p0, c, nus, mus);
-  else
-    cpml_seg_adjoint<AX, NPML, 1>(g, pf, p1, p0, c, nus, mus);
+// Fields of one layer pass. Forward: u^n, u^{n+1}, C, D (the gradient's
+// recompute), the descriptor and offset of the step (the 16-bit fields'
+// scales), and the shell receivers {x, y, z, id}, *nsrec of them. Adjoint:
+// p^{k+1}, p^k, C and the nu, mu slabs.
+struct CpmlPass {
+  const void *u;
+  void *unext;
+  const float *c;
+  float *dout;
+  const StepDesc *d;
+  int koff;
+  const int4 *srec;
+  const int *nsrec;
+  float *nus[3], *mus[3];
+};
+
+// Release and acquire over the cluster: global writes before it are visible
+// to the cluster's reads after it.
+__device__ __forceinline__ void cpml_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// A layer pass: the layer's width, the fields' storage T, and
+// whether D is updated too.
+template <int NPML_, class T, bool kStoreD>
+struct CpmlForward {
+  static constexpr int NPML = NPML_;
+  template <int AX, int SIDE, class P>
+  __device__ static __forceinline__ void line(const CpmlGeom &g, const P &pf, const CpmlPass &a,
+                                              int p, int q, const CpmlScale<T> &sc) {
+    cpml_line_forward<AX, SIDE, NPML, T, kStoreD>(g, pf, p, q,
+                                                         static_cast<const T *>(a.u),
+                                                         static_cast<T *>(a.unext), a.c, a.dout,
+                                                         sc);
+  }
+  __device__ static __forceinline__ CpmlScale<T> scale(const CpmlPass &a) {
+    CpmlScale<T> sc;
+    sc.init(a.d, a.koff);
+    return sc;
+  }
+};
+
+template <int NPML_>
+struct CpmlAdjoint {
+  static constexpr int NPML = NPML_;
+  template <int AX, int SIDE, class P>
+  __device__ static __forceinline__ void line(const CpmlGeom &g, const P &pf, const CpmlPass &a,
+                                              int p, int q, const CpmlScale<float> &) {
+    cpml_line_adjoint<AX, SIDE, NPML>(g, pf, p, q, static_cast<const float *>(a.u),
+                                             static_cast<float *>(a.unext), a.c, a.nus[AX],
+                                             a.mus[AX]);
+  }
+  __device__ static __forceinline__ CpmlScale<float> scale(const CpmlPass &) { return {}; }
+};
+
+// The lines of this CTA of cluster blk.
+template <class OP, class P>
+__device__ __forceinline__ void cpml_lines(const CpmlGeom &g, const CpmlTiles &t, const P &pf,
+                                           const CpmlPass &a, int blk) {
+  const auto sc = OP::scale(a);
+  cpml_block(
+      g, t, blk, (int)(blockIdx.x % kCpmlCluster) * kCpmlThreads + threadIdx.x,
+      [&](int ax, int side, int p, int q) {
+        if (side == 0) {
+          if (ax == 0) OP::template line<0, 0>(g, pf, a, p, q, sc);
+          else if (ax == 1) OP::template line<1, 0>(g, pf, a, p, q, sc);
+          else OP::template line<2, 0>(g, pf, a, p, q, sc);
+        } else {
+          if (ax == 0) OP::template line<0, 1>(g, pf, a, p, q, sc);
+          else if (ax == 1) OP::template line<1, 1>(g, pf, a, p, q, sc);
+          else OP::template line<2, 1>(g, pf, a, p, q, sc);
+        }
+      },
+      [] { cpml_cluster_sync(); });
+}
+
+template <class OP>
+__global__ void __cluster_dims__(kCpmlCluster, 1, 1) __launch_bounds__(kCpmlThreads, cpml_ctas(OP::NPML))
+    cpml_lines_kernel(const __grid_constant__ CpmlGeom g, const __grid_constant__ CpmlTiles t,
+                      const __grid_constant__ CpmlProf<OP::NPML> pf,
+                      const __grid_constant__ CpmlPass a) {
+  cpml_lines<OP>(g, t, pf, a, blockIdx.x / kCpmlCluster);
 }
 
 // Receivers within w of a face: {x, y, z, receiver id}, recorded from the
@@ -827,13 +1025,53 @@ __global__ void cpml_record_kernel(CpmlGeom g, const T *__restrict__ unext,
   }
 }
 
-// One served shot's layer in the shot server's batched layer launches: its
-// geometry and slabs, fields, descriptor, shell receivers, step bookkeeping
-// (batch step b0 is the shot's step 0, as in the batched sweep), and its
-// first block in each axis launch (a 1D grid that concatenates the shots'
-// blocks: ceil(lines across / 128) per row of lines).
-struct CpmlBatchShot {
+// What the host keeps of a layer to launch its passes.
+struct CpmlPlan {
   CpmlGeom g;
+  int axes;     // bit a: axis a takes the unrolled line ends
+  int variant;  // which width (cpml_variant)
+  CpmlProf<kCpmlMaxCap> prof;
+  CpmlTiles all, one[3];  // every axis at once; single axes
+};
+
+// Takes the plan's form on each axis from the grid and the layer's width
+// (g.npml set), and its tiles.
+inline void cpml_plan_forms(CpmlPlan &p) {
+  const CpmlGeom &g = p.g;
+  const int n[3] = {g.nx, g.ny, g.nz};
+  const long long fstep[3] = {1, g.pxu, (long long)g.ny * g.pxu};
+  const long long sstep[3] = {(long long)g.nz * g.ny, (long long)g.nz * g.nx,
+                              (long long)g.ny * g.nx};
+  p.axes = 0;
+  for (int ax = 0; ax < 3; ++ax)
+    if (cpml_seg_fits(g.npml, n[ax], fstep[ax], sstep[ax])) p.axes |= 1 << ax;
+  p.variant = cpml_variant(g.npml);
+  p.all = cpml_tiles(g.nx, g.ny, g.nz, g.w, -1);
+  for (int ax = 0; ax < 3; ++ax) p.one[ax] = cpml_tiles(g.nx, g.ny, g.nz, g.w, ax);
+}
+
+// Launches, enqueued on st (layer.cu): one forward step's layer terms and
+// shell receivers (store_d: also into D, no receivers), one adjoint step's.
+// a.koff and the descriptor give the step.
+void cpml_forward(int storage, bool store_d, const CpmlPlan &p, const CpmlPass &a, int sms,
+                  cudaStream_t st);
+void cpml_adjoint(const CpmlPlan &p, const CpmlPass &a, cudaStream_t st);
+
+// The unrolled line ends on tiles t of the plan (layer_lines.cuh, compiled
+// once per storage type, and for the gradient).
+template <class T, bool kStoreD>
+void cpml_launch_lines(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a,
+                       cudaStream_t st);
+void cpml_launch_adjoint_lines(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a,
+                               cudaStream_t st);
+
+// One served shot's layer in the shot server's batched layer launches: its
+// plan, fields and receivers, step bookkeeping (batch step b0 is the shot's
+// step 0, as in the batched sweep), and its first block in each launch of its
+// group (a 1D grid that concatenates the shots' blocks): 0-2 the unrolled
+// lines of every axis at once (0) or of one, 3-5 the line walks of one.
+struct CpmlBatchShot {
+  CpmlPlan plan;
   void *buf[2];  // buf[0] holds the shot's step 0
   const float *c;
   const StepDesc *desc;
@@ -841,97 +1079,23 @@ struct CpmlBatchShot {
   int nsrec;
   long long b0;
   int nsteps;
-  int blk_begin[3];
-  // per axis: 0 for the line walk, or 8 / 16 for the unrolled segment form
-  // (both faces' segments in blocks of their own), with its profile values
-  int seg[3];
-  CpmlSideProf<16> p16[3];
-  CpmlSideProf<8> p8[3];
+  int blk_begin[6];
 };
 
-__device__ __forceinline__ int cpml_batch_find(const CpmlBatchShot *shots, int nshots, int ax,
-                                               int blk) {
-  int lo = 0, hi = nshots - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (shots[mid].blk_begin[ax] <= blk) lo = mid; else hi = mid - 1;
-  }
-  return lo;
+// Launch groups: every axis unrolled (by width), some axes (by width), none.
+constexpr int kCpmlGroups = 2 * kCpmlVariants + 1;
+inline int cpml_batch_group(const CpmlPlan &p) {
+  return p.axes == 7 ? p.variant : p.axes ? kCpmlVariants + p.variant : 2 * kCpmlVariants;
 }
-
-// The axis-AX pass of batch step k over every shot of the table, each in
-// its form (shots outside their steps return at once): a shot's blocks are
-// rows x ceil(lines across / 128) for the line walk, twice that for the
-// segment form (the low face's blocks, then the high face's).
-template <int AX, class T>
-__global__ void __launch_bounds__(128, 3)
-    cpml_line_batched_kernel(const CpmlBatchShot *__restrict__ shots, int nshots, long long k) {
-  const CpmlBatchShot &sh = shots[cpml_batch_find(shots, nshots, AX, blockIdx.x)];
-  const long long n = k - sh.b0;
-  if (n < 0 || n >= sh.nsteps) return;
-  const int cur = (int)(n & 1);
-  const int across = AX == 0 ? sh.g.ny : sh.g.nx;
-  const int rows = AX == 2 ? sh.g.ny : sh.g.nz;
-  const int bpr = (across + 127) / 128;  // blocks per row of lines
-  int local = blockIdx.x - sh.blk_begin[AX];
-  const T *u = static_cast<const T *>(sh.buf[cur]);
-  T *un = static_cast<T *>(sh.buf[cur ^ 1]);
-  const int form = sh.seg[AX];
-  const int side = (form != 0 && local >= rows * bpr) ? 1 : 0;
-  local -= side * rows * bpr;
-  const int q = local / bpr;
-  const int t = (local - q * bpr) * 128 + threadIdx.x;
-  // the shot's profile values staged in shared memory (block-uniform form),
-  // read with immediate offsets where the single-grid kernels take them as
-  // constant operands
-  __shared__ CpmlSideProf<16> s16;
-  __shared__ CpmlSideProf<8> s8;
-  if (form == 16) {
-    constexpr int NV = sizeof(CpmlSideProf<16>) / 4;
-    for (int i = threadIdx.x; i < NV; i += blockDim.x)
-      reinterpret_cast<float *>(&s16)[i] = reinterpret_cast<const float *>(&sh.p16[AX])[i];
-    __syncthreads();
-    if (side == 0)
-      cpml_seg_forward<AX, 16, T, false, 0>(sh.g, s16, t, q, u, un, sh.c, nullptr, sh.desc,
-                                            (int)n);
-    else
-      cpml_seg_forward<AX, 16, T, false, 1>(sh.g, s16, t, q, u, un, sh.c, nullptr, sh.desc,
-                                            (int)n);
-  } else if (form == 8) {
-    constexpr int NV = sizeof(CpmlSideProf<8>) / 4;
-    for (int i = threadIdx.x; i < NV; i += blockDim.x)
-      reinterpret_cast<float *>(&s8)[i] = reinterpret_cast<const float *>(&sh.p8[AX])[i];
-    __syncthreads();
-    if (side == 0)
-      cpml_seg_forward<AX, 8, T, false, 0>(sh.g, s8, t, q, u, un, sh.c, nullptr, sh.desc,
-                                           (int)n);
-    else
-      cpml_seg_forward<AX, 8, T, false, 1>(sh.g, s8, t, q, u, un, sh.c, nullptr, sh.desc,
-                                           (int)n);
-  } else {
-    cpml_line_walk<AX, T, false>(sh.g, t, q, u, un, sh.c, nullptr, sh.desc, (int)n);
-  }
-}
-
-// Shell receivers of batch step k: blocks_per_shot blocks per shot (a
-// receiver plane inside the layer puts all of a shot's receivers here).
+// Blocks of a shot in launch `which` (0..5) of its group.
+int cpml_batch_blocks(const CpmlBatchShot &s, int which);
+// One batch step's launches over a group's n shots (layer.cu); blocks: their
+// totals per launch; rec_blocks: blocks per shot for its receivers.
+void cpml_batch_step(int storage, int group, const CpmlBatchShot *shots, int n,
+                     const int blocks[6], int rec_blocks, long long k, cudaStream_t st);
+// The unrolled lines of a group of one width, every axis (ax < 0) or one.
 template <class T>
-__global__ void cpml_record_batched_kernel(const CpmlBatchShot *__restrict__ shots, long long k,
-                                           int blocks_per_shot) {
-  const CpmlBatchShot &sh = shots[blockIdx.x / blocks_per_shot];
-  const int part = blockIdx.x % blocks_per_shot;
-  const long long n = k - sh.b0;
-  if (n < 0 || n >= sh.nsteps || sh.nsrec == 0) return;
-  const StepDesc *d = sh.desc;
-  CpmlScale<T> sc;
-  sc.init(d, (int)n);
-  const T *un = static_cast<const T *>(sh.buf[(n & 1) ^ 1]);
-  for (int r = part * blockDim.x + threadIdx.x; r < sh.nsrec;
-       r += blocks_per_shot * blockDim.x) {
-    const int4 e = sh.srec[r];
-    d->traces[(size_t)(d->n + n) * d->nrec + e.w] =
-        cpml_get(un + ((size_t)e.z * sh.g.ny + e.y) * sh.g.pxu + e.x, sc.so);
-  }
-}
+void cpml_launch_batched_lines(int variant, int ax, const CpmlBatchShot *shots, int n, int blocks,
+                               long long k, cudaStream_t st);
 
 }  // namespace gbw

@@ -1,0 +1,11 @@
+// The CPML layer's unrolled line ends for FP32 wavefields.
+#include "layer_lines.cuh"
+
+namespace gbw {
+
+template void cpml_launch_lines<float, false>(const CpmlPlan &, const CpmlTiles &, const CpmlPass &,
+                                           cudaStream_t);
+template void cpml_launch_batched_lines<float>(int, int, const CpmlBatchShot *, int, int, long long,
+                                            cudaStream_t);
+
+}  // namespace gbw

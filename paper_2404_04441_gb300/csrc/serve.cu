@@ -59,6 +59,14 @@ struct Group {
   StencilCoefs co;
 };
 
+// Layered shots of one storage type and one form of the layer's passes:
+// neighbours in the batch table, one launch each.
+struct LayerGroup {
+  int kind, form, first, count;
+  int blocks[6];
+  int rec_blocks;  // per shot, for its shell receivers
+};
+
 template <class C>
 Kind make_kind() {
   return Kind{C::TX,
@@ -179,11 +187,10 @@ struct serve_ctx {
   long long k = 0;  // batch steps taken
   BatchShot *d_table[kKinds] = {nullptr, nullptr, nullptr};
   std::vector<BatchShot> h_table[kKinds];
-  // layered shots per storage type: batch table and blocks per axis launch
+  // layered shots per storage type: batch table, and its launch groups
   CpmlBatchShot *d_layer[kKinds] = {nullptr, nullptr, nullptr};
   std::vector<CpmlBatchShot> h_layer[kKinds];
-  int layer_blocks[kKinds][3] = {};
-  int layer_rec_blocks[kKinds] = {1, 1, 1};  // record blocks per layered shot
+  std::vector<LayerGroup> layer_groups;
   std::vector<Group> groups;
   bool dirty = true;
   void *d_scan = nullptr;     // 16 bytes: velocity max, invalid count
@@ -244,7 +251,7 @@ int admit_layer(serve_ctx *s, Request *q, float vmax, double dt,
   const int nx = r.grid.nx, ny = r.grid.ny, nz = r.grid.nz, npml = r.npml;
   CpmlBatchShot &L = q->layer;
   L = CpmlBatchShot{};
-  CpmlGeom &g = L.g;
+  CpmlGeom &g = L.plan.g;
   g.nx = nx;
   g.ny = ny;
   g.nz = nz;
@@ -271,18 +278,16 @@ int admit_layer(serve_ctx *s, Request *q, float vmax, double dt,
     std::vector<float> hb(dims[ax]), ha(dims[ax]);
     cpml_profile(dims[ax], npml, r.reflection, r.f_cps, (double)vmax, hs[ax], dt, hb.data(),
                  ha.data());
-    const long long fstep[3] = {1, g.pxu, (long long)ny * g.pxu};
-    const long long sstep[3] = {(long long)nz * ny, (long long)nz * nx, (long long)ny * nx};
-    L.seg[ax] = cpml_seg_fits(npml, dims[ax], fstep[ax], sstep[ax]) ? npml : 0;
-    if (L.seg[ax] == 16) cpml_side_prof(hb.data(), ha.data(), dims[ax], L.p16[ax]);
-    if (L.seg[ax] == 8) cpml_side_prof(hb.data(), ha.data(), dims[ax], L.p8[ax]);
+    if (cpml_variant(npml) >= 0)
+      cpml_fill_prof(L.plan.prof, ax, hb.data(), ha.data(), dims[ax], npml);
     WAVE_TRY_CUDA(cudaMemcpyAsync((void *)g.bprof[ax], hb.data(), dims[ax] * 4,
                                   cudaMemcpyHostToDevice, st));
     WAVE_TRY_CUDA(cudaMemcpyAsync((void *)g.aprof[ax], ha.data(), dims[ax] * 4,
                                   cudaMemcpyHostToDevice, st));
     cpml_axis_coefs(g, ax, hs[ax]);
   }
-  // receivers within w of a face are re-recorded after the layer passes
+  cpml_plan_forms(L.plan);
+  // receivers within w of a face are re-recorded after the layer's terms
   std::vector<int4> shell;
   for (int i = 0; i < r.nrec; ++i) {
     const int x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
@@ -443,6 +448,7 @@ int admit(serve_ctx *s, Request *q) {
 // groups and upload the batch tables.
 int upload_tables(serve_ctx *s) {
   s->groups.clear();
+  s->layer_groups.clear();
   for (int kd = 0; kd < kKinds; ++kd) {
     std::vector<Request *> shots;
     for (Request *q : s->resident)
@@ -473,46 +479,31 @@ int upload_tables(serve_ctx *s) {
       WAVE_TRY_CUDA(cudaMemcpyAsync(s->d_table[kd], t.data(),
                                     t.size() * sizeof(BatchShot),
                                     cudaMemcpyHostToDevice, s->stream));
-    // the layered shots of this storage type: blocks of each axis launch
+    // the layered shots of this storage type, by the form of their passes
     auto &lt = s->h_layer[kd];
     lt.clear();
-    int *nb = s->layer_blocks[kd];
-    nb[0] = nb[1] = nb[2] = 0;
-    int max_srec = 0;
-    for (Request *q : shots) {
-      if (q->r.npml <= 0) continue;
-      CpmlBatchShot L = q->layer;
-      max_srec = std::max(max_srec, L.nsrec);
-      const int nx = q->r.grid.nx, ny = q->r.grid.ny, nz = q->r.grid.nz;
-      const int rows[3] = {nz, nz, ny}, across[3] = {ny, nx, nx};
-      for (int ax = 0; ax < 3; ++ax) {  // the segment form: a block set per face
-        L.blk_begin[ax] = nb[ax];
-        nb[ax] += rows[ax] * ((across[ax] + 127) / 128) * (L.seg[ax] ? 2 : 1);
+    for (int form = 0; form < kCpmlGroups; ++form) {
+      LayerGroup lg{kd, form, (int)lt.size(), 0, {}, 1};
+      for (Request *q : shots) {
+        if (q->r.npml <= 0 || cpml_batch_group(q->layer.plan) != form) continue;
+        CpmlBatchShot L = q->layer;
+        for (int i = 0; i < 6; ++i) {
+          L.blk_begin[i] = lg.blocks[i];
+          lg.blocks[i] += cpml_batch_blocks(L, i);
+        }
+        // about 256 shell receivers per record block, at most 64 blocks a shot
+        lg.rec_blocks = std::max(lg.rec_blocks, std::min(64, (L.nsrec + 255) / 256));
+        lt.push_back(L);
+        lg.count++;
       }
-      lt.push_back(L);
+      if (lg.count > 0) s->layer_groups.push_back(lg);
     }
-    // about 256 shell receivers per record block, at most 64 blocks a shot
-    s->layer_rec_blocks[kd] = std::min(64, std::max(1, (max_srec + 255) / 256));
     if (!lt.empty())
       WAVE_TRY_CUDA(cudaMemcpyAsync(s->d_layer[kd], lt.data(), lt.size() * sizeof(CpmlBatchShot),
                                     cudaMemcpyHostToDevice, s->stream));
   }
   s->dirty = false;
   return WAVE_OK;
-}
-
-// The layer passes and shell receivers of batch step k over the layered
-// shots of storage type kd.
-template <class T>
-void launch_layers(serve_ctx *s, int kd, long long k) {
-  const CpmlBatchShot *t = s->d_layer[kd];
-  const int n = (int)s->h_layer[kd].size();
-  const int *nb = s->layer_blocks[kd];
-  cpml_line_batched_kernel<0, T><<<nb[0], 128, 0, s->stream>>>(t, n, k);
-  cpml_line_batched_kernel<1, T><<<nb[1], 128, 0, s->stream>>>(t, n, k);
-  cpml_line_batched_kernel<2, T><<<nb[2], 128, 0, s->stream>>>(t, n, k);
-  const int rb = s->layer_rec_blocks[kd];
-  cpml_record_batched_kernel<T><<<n * rb, 128, 0, s->stream>>>(t, k, rb);
 }
 
 // Complete a resident shot whose steps are all done (stream synchronized).
@@ -603,12 +594,9 @@ void engine_main(serve_ctx *s) {
       for (const Group &g : s->groups)
         kind_of(g.kind).launch(g.ctas, s->stream, s->d_table[g.kind] + g.first,
                                g.count, s->k + kk, g.co);
-      if (!s->h_layer[WAVE_STORAGE_F32].empty())
-        launch_layers<float>(s, WAVE_STORAGE_F32, s->k + kk);
-      if (!s->h_layer[WAVE_STORAGE_BF16].empty())
-        launch_layers<__nv_bfloat16>(s, WAVE_STORAGE_BF16, s->k + kk);
-      if (!s->h_layer[WAVE_STORAGE_F16].empty())
-        launch_layers<__half>(s, WAVE_STORAGE_F16, s->k + kk);
+      for (const LayerGroup &lg : s->layer_groups)
+        cpml_batch_step(lg.kind, lg.form, s->d_layer[lg.kind] + lg.first, lg.count, lg.blocks,
+                        lg.rec_blocks, s->k + kk, s->stream);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);

@@ -204,13 +204,10 @@ struct wave_ctx {
   unsigned char scale_image[32];  // host staging of the 16-bit scale state
   // CPML layer (wave_set_cpml).
   bool cpml = false;
-  CpmlGeom cg{};
+  CpmlPlan cp{};
   std::vector<void *> cpml_mem;
-  DeviceBuf srec;            // receivers within w of a face: {x, y, z, id}
-  int *d_nsrec = nullptr;    // their count (device: graphs stay valid)
-  int cpml_seg_axes = 0;     // bit a: axis a runs the unrolled segment kernels
-  CpmlSideProf<8> prof8[3];  // their profile values (npml 8 or 16)
-  CpmlSideProf<16> prof16[3];
+  DeviceBuf srec;          // receivers within w of a face: {x, y, z, id}
+  int *d_nsrec = nullptr;  // their count (device: graphs stay valid)
 };
 
 namespace {
@@ -250,78 +247,29 @@ void set_coeffs(wave_ctx *c) {
   a.desc = c->d_desc;
 }
 
-// The layer's pass along axis AX of one forward step (dout: the layer's
-// term also into the stored increment D), and of one adjoint step.
-// T: the wavefields' storage; d, koff: the step's descriptor and offset
-// (the 16-bit fields' scales).
-template <int AX, class T, bool kD>
-void launch_cpml_axis(const wave_ctx *c, const CpmlGeom &g, cudaStream_t st, const T *u,
-                      T *un, float *dout, const StepDesc *d, int koff) {
-  const int inner = AX == 0 ? c->ny : c->nx, outer = AX == 2 ? c->ny : c->nz;
-  const bool seg = (c->cpml_seg_axes >> AX) & 1;
-  const dim3 grid((inner + 127) / 128, outer, seg ? 2 : 1);
-  if (!seg)
-    cpml_line_kernel<AX, T, kD><<<grid, 128, 0, st>>>(g, u, un, c->c, dout, d, koff);
-  else if (g.npml == 8)
-    cpml_seg_kernel<AX, 8, T, kD><<<grid, 128, 0, st>>>(g, c->prof8[AX], u, un, c->c, dout, d,
-                                                        koff);
-  else
-    cpml_seg_kernel<AX, 16, T, kD><<<grid, 128, 0, st>>>(g, c->prof16[AX], u, un, c->c, dout,
-                                                         d, koff);
-}
-
-// g: the context's layer, or the same layer on other memory-variable slabs
-template <class T, bool kD>
-void launch_cpml_forward(const wave_ctx *c, const CpmlGeom &g, cudaStream_t st, const T *u,
-                         T *un, float *dout, const StepDesc *d, int koff) {
-  launch_cpml_axis<0, T, kD>(c, g, st, u, un, dout, d, koff);
-  launch_cpml_axis<1, T, kD>(c, g, st, u, un, dout, d, koff);
-  launch_cpml_axis<2, T, kD>(c, g, st, u, un, dout, d, koff);
-}
-
-// One step's layer passes and shell receivers on the context's fields, in
-// their storage type.
-template <class T>
-void launch_cpml_step(const wave_ctx *c, cudaStream_t st, int cur, int koff) {
-  const T *u = static_cast<const T *>(c->buf[cur]);
-  T *un = static_cast<T *>(c->buf[cur ^ 1]);
-  launch_cpml_forward<T, false>(c, c->cg, st, u, un, nullptr, c->d_desc, koff);
-  cpml_record_kernel<T><<<c->sms, 256, 0, st>>>(c->cg, un, c->d_desc, (const int4 *)c->srec.p,
-                                               c->d_nsrec, koff);
-}
-
-template <int AX>
-void launch_cpml_adjoint_axis(const wave_ctx *c, cudaStream_t st, const float *p1, float *p0,
-                              float *nus, float *mus) {
-  const CpmlGeom &g = c->cg;
-  const int inner = AX == 0 ? c->ny : c->nx, outer = AX == 2 ? c->ny : c->nz;
-  const bool seg = (c->cpml_seg_axes >> AX) & 1;
-  const dim3 grid((inner + 127) / 128, outer, seg ? 2 : 1);
-  if (!seg)
-    cpml_adjoint_line_kernel<AX><<<grid, 128, 0, st>>>(g, p1, p0, c->c, nus, mus);
-  else if (g.npml == 8)
-    cpml_seg_adjoint_kernel<AX, 8><<<grid, 128, 0, st>>>(g, c->prof8[AX], p1, p0, c->c, nus, mus);
-  else
-    cpml_seg_adjoint_kernel<AX, 16><<<grid, 128, 0, st>>>(g, c->prof16[AX], p1, p0, c->c, nus,
-                                                          mus);
+// One forward step's layer pass on given fields.
+CpmlPass layer_pass(const wave_ctx *c, const void *u, void *un, int koff) {
+  CpmlPass a{};
+  a.u = u;
+  a.unext = un;
+  a.c = c->c;
+  a.d = c->d_desc;
+  a.koff = koff;
+  a.srec = (const int4 *)c->srec.p;
+  a.nsrec = c->d_nsrec;
+  return a;
 }
 
 // Enqueue one step on stream st: u = buf[cur], u_prev = buf[cur ^ 1]. With
-// the CPML layer: memory variables and shell points before the sweep, the
-// shell values committed after it.
+// the CPML layer: the layer's terms and the shell's receivers after the sweep.
 void enqueue_step(wave_ctx *c, cudaStream_t st, int cur, int koff) {
   SweepArgs a = c->args;
   a.unext = c->buf[cur ^ 1];
   a.koff = koff;
   c->var.launch(c->grid, st, c->tm_halo[cur], c->tm_tile[cur ^ 1], c->tm_c, a);
-  if (c->cpml) {
-    if (c->storage == WAVE_STORAGE_BF16)
-      launch_cpml_step<__nv_bfloat16>(c, st, cur, koff);
-    else if (c->storage == WAVE_STORAGE_F16)
-      launch_cpml_step<__half>(c, st, cur, koff);
-    else
-      launch_cpml_step<float>(c, st, cur, koff);
-  }
+  if (c->cpml)
+    cpml_forward(c->storage, false, c->cp, layer_pass(c, c->buf[cur], c->buf[cur ^ 1], koff),
+                 c->sms, st);
 }
 
 void drop_graphs(wave_ctx *c) {
@@ -336,18 +284,17 @@ void free_cpml(wave_ctx *c) {
   for (void *p : c->cpml_mem) cudaFree(p);
   c->cpml_mem.clear();
   c->cpml = false;
-  c->cg = CpmlGeom{};
-  c->cpml_seg_axes = 0;
+  c->cp = CpmlPlan{};
 }
 
 int zero_cpml(wave_ctx *c) {
   if (!c->cpml) return WAVE_OK;
-  const size_t sl[3] = {2ull * c->cg.npml * c->ny * c->nz,
-                        2ull * c->cg.npml * c->nz * c->nx,
-                        2ull * c->cg.npml * c->ny * c->nx};
+  const size_t sl[3] = {2ull * c->cp.g.npml * c->ny * c->nz,
+                        2ull * c->cp.g.npml * c->nz * c->nx,
+                        2ull * c->cp.g.npml * c->ny * c->nx};
   for (int ax = 0; ax < 3; ++ax) {
-    WAVE_TRY_CUDA(cudaMemsetAsync(c->cg.psi[ax], 0, sl[ax] * 4, c->stream));
-    WAVE_TRY_CUDA(cudaMemsetAsync(c->cg.zeta[ax], 0, sl[ax] * 4, c->stream));
+    WAVE_TRY_CUDA(cudaMemsetAsync(c->cp.g.psi[ax], 0, sl[ax] * 4, c->stream));
+    WAVE_TRY_CUDA(cudaMemsetAsync(c->cp.g.zeta[ax], 0, sl[ax] * 4, c->stream));
   }
   return WAVE_OK;
 }
@@ -952,7 +899,7 @@ int propagate_begin(wave_ctx *c, const wave_shot *shot, int nsteps,
     WAVE_TRY_CUDA(cudaMemsetAsync(c->d_nsrec, 0, sizeof(int), st));
     if (nrec > 0) {
       rec_shell_kernel<<<std::min(c->sms * 4, (nrec + 255) / 256), 256, 0, st>>>(
-          drec, nrec, geom, c->cg.w, (int4 *)c->srec.p, c->d_nsrec);
+          drec, nrec, geom, c->cp.g.w, (int4 *)c->srec.p, c->d_nsrec);
       WAVE_TRY_CUDA(cudaGetLastError());
     }
   }
@@ -1194,7 +1141,7 @@ int wave_set_cpml(wave_ctx *c, int npml, double R, double f_cps) {
     if (c->ny > 65535 || c->nz > 65535) return WAVE_ENOTSUP;
     WAVE_TRY_CUDA(cudaStreamSynchronize(c->stream));
     free_cpml(c);
-    CpmlGeom &g = c->cg;
+    CpmlGeom &g = c->cp.g;
     g.nx = c->nx;
     g.ny = c->ny;
     g.nz = c->nz;
@@ -1224,25 +1171,15 @@ int wave_set_cpml(wave_ctx *c, int npml, double R, double f_cps) {
       // Profiles (FP64, stored FP32) and derivative coefficients.
       std::vector<float> hb(dims[ax]), ha(dims[ax]);
       cpml_profile(dims[ax], npml, R, f_cps, c->vmax, hs[ax], c->dt, hb.data(), ha.data());
-      // the unrolled segment kernels where they apply (cpml_seg_fits), with
-      // the field and slab steps along the axis (the wavefields' pitch is at
-      // least that of v^2 dt^2)
-      const long long fstep[3] = {1, c->pxu, (long long)c->ny * c->pxu};
-      const long long sstep[3] = {(long long)c->nz * c->ny, (long long)c->nz * c->nx,
-                                  (long long)c->ny * c->nx};
-      if (cpml_seg_fits(npml, dims[ax], fstep[ax], sstep[ax])) {
-        c->cpml_seg_axes |= 1 << ax;
-        if (npml == 8)
-          cpml_side_prof(hb.data(), ha.data(), dims[ax], c->prof8[ax]);
-        else
-          cpml_side_prof(hb.data(), ha.data(), dims[ax], c->prof16[ax]);
-      }
+      if (cpml_variant(npml) >= 0)
+        cpml_fill_prof(c->cp.prof, ax, hb.data(), ha.data(), dims[ax], npml);
       WAVE_TRY_CUDA(cudaMemcpy((void *)g.bprof[ax], hb.data(), dims[ax] * 4,
                                cudaMemcpyHostToDevice));
       WAVE_TRY_CUDA(cudaMemcpy((void *)g.aprof[ax], ha.data(), dims[ax] * 4,
                                cudaMemcpyHostToDevice));
       cpml_axis_coefs(g, ax, hs[ax]);
     }
+    cpml_plan_forms(c->cp);
     if (!c->d_nsrec) WAVE_TRY_CUDA(cudaMalloc((void **)&c->d_nsrec, sizeof(int)));
     WAVE_TRY_CUDA(cudaMemset(c->d_nsrec, 0, sizeof(int)));
     c->cpml = true;
@@ -1472,7 +1409,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   // With the CPML layer: the memory variables psi, zeta (per axis) are saved
   // with each checkpoint, the recompute steps the saved copies in place, and
   // the adjoint carries its nu, mu slabs.
-  const CpmlGeom &cg = c->cg;
+  const CpmlGeom &cg = c->cp.g;
   size_t sl[3] = {0, 0, 0};
   float *ckpt_l = nullptr, *nus[3] = {}, *mus[3] = {};
   if (c->cpml) {
@@ -1486,18 +1423,20 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   }
   // the layer slabs held by a segment's checkpoint (per axis psi, then zeta)
   auto layer_of = [&](int sgm) {
-    CpmlGeom gg = cg;
+    CpmlPlan pl = c->cp;
+    CpmlGeom &gg = pl.g;
     float *q = ckpt_l + (sl[0] + sl[1] + sl[2]) * 2 * sgm;
     for (int ax = 0; ax < 3; ++ax) {
       gg.psi[ax] = q;
       gg.zeta[ax] = q + sl[ax];
       q += 2 * sl[ax];
     }
-    return gg;
+    return pl;
   };
   // copies the context's memory variables into a segment's checkpoint
   auto layer_ckpt = [&](int sgm, cudaStream_t cs) -> int {
-    const CpmlGeom gg = layer_of(sgm);
+    const CpmlPlan pl = layer_of(sgm);
+    const CpmlGeom &gg = pl.g;
     for (int ax = 0; ax < 3; ++ax) {
       WAVE_TRY_CUDA(cudaMemcpyAsync(gg.psi[ax], cg.psi[ax], sl[ax] * 4,
                                     cudaMemcpyDeviceToDevice, cs));
@@ -1574,7 +1513,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
       const int me = field_maps(rbuf[b], &rhalo[b], &rtile[b]);
       if (me) return me;
     }
-    const CpmlGeom rg = c->cpml ? layer_of(sgm) : cg;
+    const CpmlPlan rp = c->cpml ? layer_of(sgm) : c->cp;
     int cur = 0;
     for (int n = s0; n < s1; ++n) {
       SweepArgs a = args_d;
@@ -1583,9 +1522,11 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
       a.unext = rbuf[cur ^ 1];
       a.dout = dslot + (size_t)(n - s0) * fe;
       launch_mode<kModeStoreD>(c, rs, grid_d, rhalo[cur], rtile[cur ^ 1], a);
-      if (c->cpml)  // the layer's terms, into u^{n+1} and D^n
-        launch_cpml_forward<float, true>(c, rg, rs, rbuf[cur], rbuf[cur ^ 1], a.dout, nullptr,
-                                         0);
+      if (c->cpml) {  // the layer's terms, into u^{n+1} and D^n
+        CpmlPass lp = layer_pass(c, rbuf[cur], rbuf[cur ^ 1], 0);
+        lp.dout = a.dout;
+        cpml_forward(c->storage, true, rp, lp, c->sms, rs);
+      }
       cur ^= 1;
     }
     if (nslot == 2) WAVE_TRY_CUDA(cudaEventRecord(gs.rec_done[sgm & 1], rs));
@@ -1668,11 +1609,12 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
     else
       launch_mode<kModeInject>(c, st, grid_a, ahalo[ca], atile[ca ^ 1], a);
     if (c->cpml) {  // the layer's adjoint terms, from p^{k+1} into p^k
-      const float *p1 = padj[ca];
-      float *p0 = padj[ca ^ 1];
-      launch_cpml_adjoint_axis<0>(c, st, p1, p0, nus[0], mus[0]);
-      launch_cpml_adjoint_axis<1>(c, st, p1, p0, nus[1], mus[1]);
-      launch_cpml_adjoint_axis<2>(c, st, p1, p0, nus[2], mus[2]);
+      CpmlPass lp = layer_pass(c, padj[ca], padj[ca ^ 1], 0);
+      for (int ax = 0; ax < 3; ++ax) {
+        lp.nus[ax] = nus[ax];
+        lp.mus[ax] = mus[ax];
+      }
+      cpml_adjoint(c->cp, lp, st);
     }
     if (dsrc && k % kGradFold == 0)
       grad_fold_kernel<<<c->sms * 4, 256, 0, st>>>(gacc, ghi, glo, (long long)(fe / 4));
