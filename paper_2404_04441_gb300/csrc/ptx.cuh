@@ -87,7 +87,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar,
 // threads that still poll give up as soon as they see it.
 __device__ __forceinline__ void mbar_wait_or_flag(uint32_t bar, uint32_t parity,
                                                   uint64_t limit_ns, volatile int *failed) {
-  if (mbar_try_wait_s(bar, parity)) return;
+  if (__builtin_expect(mbar_try_wait_s(bar, parity), 1)) return;
   const uint64_t t0 = global_timer_ns();
   for (uint32_t i = 1; i < (1u << 28); ++i) {
     if (mbar_try_wait_s(bar, parity)) return;

@@ -276,10 +276,10 @@ struct TcCfg {
   static constexpr uint32_t U_BYTES = U_SLOT * sizeof(T);
   static constexpr uint32_t UP_BYTES = P_SLOT * sizeof(T);
   static constexpr uint32_t C_BYTES = P_SLOT * 4;
-  // rings, then one barrier per stage in flight (receivers are recorded
-  // by the threads that own the points: no staging plane)
+  // rings, the receivers' two staging planes, one barrier per stage in flight
   static constexpr size_t SMEM_BYTES = (size_t)SU * U_BYTES +
-                                       (size_t)SP * (UP_BYTES + C_BYTES) + NB * 8 + 8;
+                                       (size_t)SP * (UP_BYTES + C_BYTES) + 2 * TX * TY * 4 +
+                                       NB * 8 + 8;
   static_assert(SU == 9, "the plane loop keeps ring slot = plane mod 9");
   static_assert(U_BYTES % 128 == 0 && UP_BYTES % 128 == 0 && C_BYTES % 128 == 0,
                 "slot alignment");
@@ -299,14 +299,27 @@ __device__ __forceinline__ void acc_exact(float &hi, float &lo, float u, float d
   lo = __fadd_rn(lo, __fadd_rn(err, e));
 }
 
-// First entry of e[lo, hi), sorted by depth .x, at depth zb or deeper. A
-// binary search: a walk from lo costs a dependent load per entry (32 a tile
-// with receivers every 4th point), in every CTA below the receiver plane.
-__device__ __forceinline__ int first_at_depth(const int4 *e, int lo, int hi, int zb) {
-  if (zb == 0) return lo;
+// Entries of e[lo, hi), sorted by depth .x, that satisfy take(entry), which
+// holds for the first n of them: each thread asks its own, all learn n (block
+// barriers). One load latency for up to N entries; walking them one by one
+// costs a dependent load each in every thread, which took 4 us of a 64^3 step
+// (32 receivers in a tile): 7.9 -> 4.6 us, 48.9 -> 44.5 at 256^3.
+template <int N, class F>
+__device__ __forceinline__ int leading_entries(const int4 *e, int lo, int hi, F take) {
+  const int beg = lo;
+  for (;;) {
+    const int i = lo + threadIdx.x;
+    const int n = __syncthreads_count(i < hi && take(e[i]));
+    lo += n;
+    if (n < N) return lo - beg;
+  }
+}
+
+// First entry of e[lo, hi), sorted by depth .x, deeper than j.
+__device__ __forceinline__ int first_below(const int4 *e, int lo, int hi, int j) {
   while (lo < hi) {
     const int mid = lo + ((hi - lo) >> 1);
-    if (e[mid].x < zb) lo = mid + 1; else hi = mid;
+    if (e[mid].x <= j) lo = mid + 1; else hi = mid;
   }
   return lo;
 }
@@ -402,7 +415,8 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
     const int tile = by * a.ntx + bx;
     rcur = d->rec_start[tile];
     rend = d->rec_start[tile + 1];
-    rcur = first_at_depth(rec, rcur, rend, zb);
+    if (zb > 0)
+      rcur += leading_entries<C::THREADS>(rec, rcur, rend, [&](const int4 &r4) { return r4.x < zb; });
   }
   int rz = (rcur < rend) ? rec[rcur].x : 0x7fffffff;  // z of the next receiver
   float *trow = (nrec > 0) ? d->traces + (size_t)n * nrec : nullptr;
@@ -416,7 +430,9 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       irow = d->inj_val + (size_t)n * d->ninj;
       icur = d->inj_start[tile];
       iend = d->inj_start[tile + 1];
-      icur = first_at_depth(inj, icur, iend, zb);
+      if (zb > 0)
+        icur += leading_entries<C::THREADS>(inj, icur, iend,
+                                            [&](const int4 &r4) { return r4.x < zb; });
       if (icur < iend) iz = inj[icur].x;
     }
   }
@@ -517,7 +533,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       // the failed stage's slot could be issued again.
       mbar_wait_or_flag(bars_s + 8u * (s % C::NB), (s / C::NB) & 1, kWaitLimitNs, failed);
       __syncthreads();
-      if (i % 3 == 0 && *failed) goto wait_failed;
+      if (i % 3 == 0 && __builtin_expect(*failed, 0)) goto wait_failed;
       if (tid == 0 && s + C::PF < NS) issue(s + C::PF);
       // Front plane (j+4) into the queue.
       const int fslot = (C::SU == 9) ? p : (s % C::SU);
@@ -651,7 +667,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
           const float2 dl = __fmul2_rn(cvl, lo), dh = __fmul2_rn(cvh, hi);
           dv = make_float4(dl.x, dl.y, dh.x, dh.y);
         }
-        if (src_here && j == sz && sy == ty * C::VY + v) {
+        if (__builtin_expect(src_here && j == sz && sy == ty * C::VY + v, 0)) {
           const int e = sx - 4 * tx;
           if (e == 0) o.x = fmaf(cv.x, wsrc, o.x);
           if (e == 1) o.y = fmaf(cv.y, wsrc, o.y);
@@ -675,25 +691,22 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       // Point injections on this plane (adjoint sources): stage the plane,
       // add v^2 dt^2 * value per entry (repeated points add up), read back.
       if constexpr ((kMode & kModeInject) != 0) {
-        if (j == iz) {
+        if (__builtin_expect(j == iz, 0)) {
 #pragma unroll
           for (int v = 0; v < C::VY; ++v)
             *reinterpret_cast<float4 *>(sr + (ty * C::VY + v) * C::TX + 4 * tx) =
                 res[v];
           __syncthreads();
-          int last = icur;
-          while (last < iend && inj[last].x == j) ++last;
-          for (int e = icur + tid; e < last; e += C::THREADS) {
-            const int4 r4 = inj[e];
+          icur += leading_entries<C::THREADS>(inj, icur, iend, [&](const int4 &r4) {
+            if (r4.x != j) return false;
             atomicAdd(&sr[r4.y], pc[r4.y] * irow[r4.z]);
-          }
-          __syncthreads();
+            return true;
+          });  // ends with a barrier: the sums are complete
 #pragma unroll
           for (int v = 0; v < C::VY; ++v)
             res[v] = *reinterpret_cast<const float4 *>(
                 sr + (ty * C::VY + v) * C::TX + 4 * tx);
           __syncthreads();  // the staging plane is free again
-          icur = last;
           iz = (icur < iend) ? inj[icur].x : 0x7fffffff;
         }
       }
@@ -725,7 +738,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       if constexpr ((kMode & kModeGradAcc) != 0) grad_load(j + 1);
 
       // Receivers on this plane: stage the plane, then one thread per entry.
-      if (j == rz) {
+      if (__builtin_expect(j == rz, 0)) {
 #pragma unroll
         for (int v = 0; v < C::VY; ++v) {
           float4 t = res[v];
@@ -739,13 +752,10 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
               t;
         }
         __syncthreads();
-        int last = rcur;
-        while (last < rend && rec[last].x == j) ++last;
-        for (int e = rcur + tid; e < last; e += C::THREADS) {
-          const int4 r4 = rec[e];
-          trow[r4.z] = sr[r4.y];
-        }
-        rcur = last;
+        rcur += leading_entries<C::THREADS>(rec, rcur, rend, [&](const int4 &r4) {
+          if (r4.x == j) trow[r4.z] = sr[r4.y];
+          return r4.x == j;
+        });
         rz = (rcur < rend) ? rec[rcur].x : 0x7fffffff;
       }
     }
@@ -856,14 +866,15 @@ __device__ __forceinline__ float2 pair_to_f32<__nv_bfloat16>(unsigned w) {
   return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
 
+// 5040 w_|off| (kWInt) as selects: as a switch, the 24 calls below branched
+// lane by lane and took 7 k of the 9 k cycles a CTA needed to its first plane:
+// with the receivers' change 0.989 -> 0.920 ms a step at 1024 x 1024 x 512.
 __device__ __forceinline__ float wint(int off) {
-  switch (off < 0 ? -off : off) {
-    case 1: return 8064.f;   // 5040 w_m, m = 1..4 (kWInt)
-    case 2: return -1008.f;
-    case 3: return 128.f;
-    case 4: return -9.f;
-    default: return 0.f;
-  }
+  const int m = off < 0 ? -off : off;
+  float w = m == 1 ? 8064.f : 0.f;
+  w = m == 2 ? -1008.f : w;
+  w = m == 3 ? 128.f : w;
+  return m == 4 ? -9.f : w;
 }
 
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) {
@@ -886,7 +897,8 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
   T *sp = reinterpret_cast<T *>(base + C::SU * C::U_BYTES);
   float *sc = reinterpret_cast<float *>(base + C::SU * C::U_BYTES +
                                         C::SP * C::UP_BYTES);
-  uint64_t *bars = reinterpret_cast<uint64_t *>(sc + C::SP * C::P_SLOT);
+  float *sr = sc + C::SP * C::P_SLOT;  // receiver staging (two planes)
+  uint64_t *bars = reinterpret_cast<uint64_t *>(sr + 2 * C::TX * C::TY);
   volatile int *failed = reinterpret_cast<volatile int *>(bars + C::NB);
 
   const int tid = threadIdx.x;
@@ -942,7 +954,8 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
     const int tile = by * a.ntx + bx;
     rcur = d->rec_start[tile];
     rend = d->rec_start[tile + 1];
-    rcur = first_at_depth(rec, rcur, rend, zb);
+    if (zb > 0)
+      rcur += leading_entries<C::THREADS>(rec, rcur, rend, [&](const int4 &r4) { return r4.x < zb; });
   }
   int rz = (rcur < rend) ? rec[rcur].x : 0x7fffffff;
   float *trow = (nrec > 0) ? d->traces + (size_t)n * nrec : nullptr;
@@ -982,17 +995,22 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
 #pragma unroll
   for (int ks = 0; ks < 2; ++ks) {
     auto A = [&](int m, int k) {
-      return ks == 0 ? wint(k - 4 - m) : (k >= 8 ? wint(k + 4 - m) : 0.f);
+      const float w = wint(ks == 0 ? k - 4 - m : k + 4 - m);
+      return ks == 0 || k >= 8 ? w : 0.f;
     };
     ya[ks][0] = pack_pair<T>(A(g, 2 * cq), A(g, 2 * cq + 1));
     ya[ks][1] = pack_pair<T>(A(g + 8, 2 * cq), A(g + 8, 2 * cq + 1));
     ya[ks][2] = pack_pair<T>(A(g, 2 * cq + 8), A(g, 2 * cq + 9));
     ya[ks][3] = pack_pair<T>(A(g + 8, 2 * cq + 8), A(g + 8, 2 * cq + 9));
     auto B = [&](int k, int nn) {
-      return ks == 0 ? wint(k - 8 - nn) : (k >= 8 ? wint(k - nn) : 0.f);
+      const float w = wint(ks == 0 ? k - 8 - nn : k - nn);
+      return ks == 0 || k >= 8 ? w : 0.f;
     };
     xbw[ks][0] = pack_pair<T>(B(2 * cq, g), B(2 * cq + 1, g));
     xbw[ks][1] = pack_pair<T>(B(2 * cq + 8, g), B(2 * cq + 9, g));
+    // opaque: kept in registers, not formed again in the plane loop
+    asm volatile("" : "+r"(ya[ks][0]), "+r"(ya[ks][1]), "+r"(ya[ks][2]), "+r"(ya[ks][3]),
+                 "+r"(xbw[ks][0]), "+r"(xbw[ks][1]));
   }
   // ldmatrix row addresses within a u slot (elements). y (transposed): lane
   // l gives row (l & 7) of matrix l / 8 = slot rows 0..7, 8..15, 8..15,
@@ -1012,9 +1030,9 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
   // the thread's points in a u slot and in a tile slot (elements)
   const int ua = (g + kR) * C::UW + C::HX + xt, ub = ua + 8 * C::UW;
   const int pa = g * C::PW + xt, pb = pa + 8 * C::PW;
-  // their indices within the tile (receiver table entries) and in the
-  // output field (elements of plane 0), with their bounds
+  // their indices within the tile (receiver table entries)
   const int la = g * C::TX + xt, lb = la + 8 * C::TX;
+  // their index in the output field (elements of plane 0), with its bounds
   const size_t plane_stride = (size_t)a.ny * a.px;
   const size_t oa = (size_t)(y0 + g) * a.px + (x0 + xt);
   const size_t ob = oa + 8 * (size_t)a.px;
@@ -1030,6 +1048,19 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
   float4 q[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) q[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+
+  // records the receivers of a staged plane, one thread per entry; two staging
+  // planes by turns, so the next plane can be staged meanwhile
+  auto record = [&](int jr) {
+    const float *st = sr + (jr & 1) * C::TX * C::TY;
+    const int end = first_below(rec, rcur, rend, jr);
+    for (int e = rcur + tid; e < end; e += C::THREADS) {
+      const int4 r4 = rec[e];
+      trow[r4.z] = st[r4.y];
+    }
+    rcur = end;
+    rz = (rcur < rend) ? rec[rcur].x : 0x7fffffff;
+  };
 
   // the 8 u-only stages (see sweep_cta)
   int s = 0;
@@ -1060,8 +1091,11 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
       // wait that gave up is looked for every third plane (see sweep_cta).
       mbar_wait_or_flag(bars_s + 8u * p, i == 0 ? par9 : par9 ^ 1u, kWaitLimitNs, failed);
       __syncthreads();
-      if (i % 3 == 0 && *failed) goto wait_failed;
+      if (i % 3 == 0 && __builtin_expect(*failed, 0)) goto wait_failed;
       if (tid == 0 && s < ns_issue) issue(s + C::PF, (p + C::PF) % 9);
+      // The last plane's receivers: no barrier of their own, which in this
+      // loop, even where no receiver is, cost 100 cycles of 710 a plane.
+      if (__builtin_expect(zb - 2 * kR + s - 1 == rz, 0)) record(rz);
       {
         const T *uf = su + p * C::U_SLOT;  // SU == 9: slot of stage s is s % 9
         const float2 fa = pair_to_f32<T>(*reinterpret_cast<const unsigned *>(uf + ua));
@@ -1115,7 +1149,7 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
                                __fmul2_rn(s2v, make_float2(-upa.x, -upa.y)));
         float2 oh = __ffma2_rn(s1v, __ffma2_rn(cvh, hi, __fadd2_rn(uh, uh)),
                                __fmul2_rn(s2v, make_float2(-upb.x, -upb.y)));
-        if (j == src_j) {
+        if (__builtin_expect(j == src_j, 0)) {
           const int e = sx - xt;
           if (sy == g) {
             if (e == 0) ol.x = fmaf(cvl.x, wsrc, ol.x);
@@ -1132,24 +1166,19 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
         if (wb) __stcs(reinterpret_cast<unsigned *>(outb), pack_pair<T>(oh.x, oh.y));
         outa += plane_stride;
         outb += plane_stride;
-        // Receivers on this plane: each thread records the entries at its
-        // own points (no staging, so no barrier across the warps).
-        if (j == rz) {
-          int e = rcur;
-          for (; e < rend; ++e) {
-            const int4 r4 = rec[e];
-            if (r4.x != j) break;
-            const int da = r4.y - la, db = r4.y - lb;
-            if (da == 0) trow[r4.z] = ol.x * so;
-            if (da == 1) trow[r4.z] = ol.y * so;
-            if (db == 0) trow[r4.z] = oh.x * so;
-            if (db == 1) trow[r4.z] = oh.y * so;
-          }
-          rcur = e;
-          rz = (rcur < rend) ? rec[rcur].x : 0x7fffffff;
+        // Receivers on this plane: staged here, recorded past the next
+        // plane's barrier.
+        if (__builtin_expect(j == rz, 0)) {
+          float *st = sr + (j & 1) * C::TX * C::TY;
+          *reinterpret_cast<float2 *>(st + la) = make_float2(ol.x * so, ol.y * so);
+          *reinterpret_cast<float2 *>(st + lb) = make_float2(oh.x * so, oh.y * so);
         }
       }
     }
+  }
+  if (rz == ze - 1) {  // receivers on the last plane
+    __syncthreads();
+    record(rz);
   }
   {
 #pragma unroll
