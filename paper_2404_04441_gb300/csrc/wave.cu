@@ -953,20 +953,55 @@ static int field_slot(const wave_ctx *c, int which) {
   return (int)((c->step + (which ? 3 : 0)) & 3);
 }
 
+// Rows of a field between the caller's packed array (nx floats a row) and the
+// context's pitched one, by kernel.
 template <class T>
-static void launch_from_stored(const wave_ctx *c, float *dst, const void *src,
-                               int slot) {
-  from_stored_kernel<T><<<c->sms * 4, 256, 0, c->stream>>>(
-      dst, reinterpret_cast<const T *>(src), c->pxu, c->nx,
-      (long long)c->ny * c->nz, c->d_desc, slot);
+static void launch_from_stored(const wave_ctx *c, float *dst, const void *src, int slot) {
+  const long long rows = (long long)c->ny * c->nz;
+  const int v = rows_of_float4(dst, c->nx) ? 4 : 1;
+  const RowLaunch l = row_launch(c->nx, rows, v, c->sms);
+  const T *f = reinterpret_cast<const T *>(src);
+  if (v == 4)
+    from_stored_kernel<T, 4><<<l.grid, l.block, 0, c->stream>>>(dst, f, c->pxu, c->nx, rows,
+                                                                c->d_desc, slot);
+  else
+    from_stored_kernel<T, 1><<<l.grid, l.block, 0, c->stream>>>(dst, f, c->pxu, c->nx, rows,
+                                                                c->d_desc, slot);
 }
 
 template <class T>
-static void launch_to_stored(const wave_ctx *c, void *dst, const float *src,
-                             int slot) {
-  to_stored_kernel<T><<<c->sms * 4, 256, 0, c->stream>>>(
-      reinterpret_cast<T *>(dst), c->pxu, src, c->nx,
-      (long long)c->ny * c->nz, c->d_desc, slot);
+static void launch_to_stored(const wave_ctx *c, void *dst, const float *src, int slot) {
+  const long long rows = (long long)c->ny * c->nz;
+  const int v = rows_of_float4(src, c->nx) ? 4 : 1;
+  const RowLaunch l = row_launch(c->nx, rows, v, c->sms);
+  T *f = reinterpret_cast<T *>(dst);
+  if (v == 4)
+    to_stored_kernel<T, 4><<<l.grid, l.block, 0, c->stream>>>(f, c->pxu, src, c->nx, rows,
+                                                              c->d_desc, slot);
+  else
+    to_stored_kernel<T, 1><<<l.grid, l.block, 0, c->stream>>>(f, c->pxu, src, c->nx, rows,
+                                                              c->d_desc, slot);
+}
+
+// An FP32 field's rows to (out) or from (in) the caller's packed array: by
+// kernel in the device's own memory, by copy engine elsewhere.
+static int copy_field(const wave_ctx *c, float *dst, long long dpitch, const float *src,
+                      long long spitch, const float *user) {
+  const long long rows = (long long)c->ny * c->nz;
+  if (!is_memory_of(user, c->device)) {
+    WAVE_TRY_CUDA(cudaMemcpy2DAsync(dst, (size_t)dpitch * 4, src, (size_t)spitch * 4,
+                                    (size_t)c->nx * 4, (size_t)rows, cudaMemcpyDefault,
+                                    c->stream));
+    return WAVE_OK;
+  }
+  const int v = rows_of_float4(user, c->nx) ? 4 : 1;
+  const RowLaunch l = row_launch(c->nx, rows, v, c->sms);
+  if (v == 4)
+    copy_rows_kernel<4><<<l.grid, l.block, 0, c->stream>>>(dst, dpitch, src, spitch, c->nx, rows);
+  else
+    copy_rows_kernel<1><<<l.grid, l.block, 0, c->stream>>>(dst, dpitch, src, spitch, c->nx, rows);
+  WAVE_TRY_CUDA(cudaGetLastError());
+  return WAVE_OK;
 }
 
 extern "C" {
@@ -976,10 +1011,8 @@ int wave_get_field(const wave_ctx *c, int which, float *out) {
   const void *src = c->buf[which == 0 ? c->cur : (c->cur ^ 1)];
   const bool host_out = !is_device_ptr(out);
   if (c->storage == WAVE_STORAGE_F32) {
-    WAVE_TRY_CUDA(cudaMemcpy2DAsync(out, (size_t)c->nx * 4, src,
-                                    (size_t)c->px * 4, (size_t)c->nx * 4,
-                                    (size_t)c->ny * c->nz, cudaMemcpyDefault,
-                                    c->stream));
+    const int st = copy_field(c, out, c->nx, static_cast<const float *>(src), c->px, out);
+    if (st) return st;
     if (host_out) return read_device_error(const_cast<wave_ctx *>(c));
     return WAVE_OK;
   }
@@ -1034,7 +1067,8 @@ static int set_state_16(wave_ctx *c, const float *u, const float *u_prev,
     unsigned *dm = reinterpret_cast<unsigned *>(c->d_scratch);
     cudaError_t e = cudaMemsetAsync(dm, 0, 8, st);
     for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
-      absmax_kernel<<<c->sms * 4, 256, 0, st>>>(src[b], (long long)n, dm + b);
+      absmax_kernel<<<c->sms * 4, 256, 0, st>>>(
+          src[b], (long long)n, reinterpret_cast<uintptr_t>(src[b]) % 16 == 0, dm + b);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess)
@@ -1090,11 +1124,10 @@ int wave_set_state(wave_ctx *c, const float *u, const float *u_prev,
   if (c->storage != WAVE_STORAGE_F32) return set_state_16(c, u, u_prev, step);
   c->cur = 0;
   const float *src[2] = {u, u_prev};
-  for (int b = 0; b < 2; ++b)
-    WAVE_TRY_CUDA(cudaMemcpy2DAsync(c->buf[b], (size_t)c->px * 4, src[b],
-                                    (size_t)c->nx * 4, (size_t)c->nx * 4,
-                                    (size_t)c->ny * c->nz, cudaMemcpyDefault,
-                                    c->stream));
+  for (int b = 0; b < 2; ++b) {
+    const int st = copy_field(c, static_cast<float *>(c->buf[b]), c->px, src[b], c->nx, src[b]);
+    if (st) return st;
+  }
   c->step = step;
   int zs = zero_cpml(c);
   if (zs) return zs;
