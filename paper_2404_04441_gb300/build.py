@@ -16,7 +16,8 @@ LIB = os.path.join(OUT_DIR, "libgbwave.so")
 SOURCES = [os.path.join(CSRC, f) for f in (
     "wave.cu", "serve.cu", "layer.cu", "layer_f32.cu", "layer_f16.cu", "layer_bf16.cu",
     "layer_grad.cu")]
-DEPS = SOURCES + [os.path.join(CSRC, f) for f in ("sweep.cuh", "ptx.cuh", "common.cuh", "cpml.cuh", "layer_lines.cuh")] + [
+DEPS = SOURCES + [os.path.join(CSRC, f) for f in (
+    "sweep.cuh", "ptx.cuh", "common.cuh", "cpml.cuh", "layer_lines.cuh", "workspace.cuh")] + [
     os.path.join(ROOT, "include", f) for f in ("wave.h", "wave_serve.h")]
 
 NVCC_FLAGS = [

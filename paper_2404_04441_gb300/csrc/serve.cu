@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "cpml.cuh"
 #include "sweep.cuh"
+#include "workspace.cuh"
 
 using namespace gbw;
 
@@ -208,8 +209,13 @@ namespace {
 int serve_alloc(serve_ctx *s, void **p, size_t bytes) {
   *p = nullptr;
   if (s->fault_alloc >= 0 && s->allocs++ == s->fault_alloc) return WAVE_ENOMEM;
-  WAVE_TRY_CUDA(cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 256), s->pool, s->stream));
-  return WAVE_OK;
+  bytes = std::max<size_t>(bytes, 256);
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, s->pool, s->stream);
+  if (e == cudaErrorMemoryAllocation && drop_kept_workspace(s->device)) {
+    cudaGetLastError();
+    e = cudaMallocFromPoolAsync(p, bytes, s->pool, s->stream);
+  }
+  return cuda_status(e);
 }
 
 void release(serve_ctx *s, Request *q) {
@@ -707,13 +713,13 @@ int serve_create(size_t hbm_budget_bytes, int max_slots, void *stream,
     e = cuda_status(cudaFuncSetAttribute(
         k.func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
     if (e == WAVE_OK)
-      e = cuda_status(cudaMalloc((void **)&s->d_table[kd],
+      e = cuda_status(device_malloc((void **)&s->d_table[kd],
                                  sizeof(BatchShot) * (size_t)max_slots));
     if (e == WAVE_OK)
-      e = cuda_status(cudaMalloc((void **)&s->d_layer[kd],
+      e = cuda_status(device_malloc((void **)&s->d_layer[kd],
                                  sizeof(CpmlBatchShot) * (size_t)max_slots));
   }
-  if (e == WAVE_OK) e = cuda_status(cudaMalloc(&s->d_scan, 16));
+  if (e == WAVE_OK) e = cuda_status(device_malloc(&s->d_scan, 16));
   if (e == WAVE_OK) {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;

@@ -14,12 +14,14 @@
 #include <functional>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/wave.h"
 #include "common.cuh"
 #include "cpml.cuh"
 #include "sweep.cuh"
+#include "workspace.cuh"
 
 using namespace gbw;
 
@@ -164,6 +166,7 @@ struct wave_ctx {
   cudaStream_t stream = nullptr;
   cudaStream_t capture_stream = nullptr;
   int device = 0;
+  bool counted = false;  // among its device's contexts (KeptWork)
   void *base = nullptr;  // one allocation: both wavefields, c, desc, scratch
   void *buf[2] = {nullptr, nullptr};  // buf[cur] = u, buf[cur ^ 1] = u_prev
   float *c = nullptr;
@@ -210,9 +213,75 @@ struct wave_ctx {
   int *d_nsrec = nullptr;  // their count (device: graphs stay valid)
 };
 
+// The gradient's workspace, kept between calls: one block per device, of at
+// most 1/16 of its memory, while a context lives there. Mapping and unmapping
+// it on each call cost 4.1 ms of a gradient at 256^3 x 160 steps (6.3 GB in 14
+// allocations; 36.4 -> 31.1 ms) and a call of one step 3.8 ms. A call takes
+// the block out, so calls that run at once (other threads, other streams) have
+// blocks of their own, and gives it back after its last stream synchronisation;
+// what does not fit, or a second block, is freed. An allocation of the library
+// that fails frees the kept block and tries again; so does the end of the last
+// context.
+namespace {
+
+constexpr int kWorkDevices = 64;
+
+struct KeptWork {
+  std::mutex mu;
+  void *p[kWorkDevices] = {};
+  size_t cap[kWorkDevices] = {};
+  int contexts[kWorkDevices] = {};
+};
+KeptWork g_work;
+
+// Frees a device's kept block (mu held).
+bool drop_locked(int dev) {
+  if (!g_work.p[dev]) return false;
+  cudaFree(g_work.p[dev]);
+  g_work.p[dev] = nullptr;
+  g_work.cap[dev] = 0;
+  return true;
+}
+
+void count_context(int dev, int by) {
+  if (dev < 0 || dev >= kWorkDevices) return;
+  std::lock_guard<std::mutex> lock(g_work.mu);
+  if ((g_work.contexts[dev] += by) == 0) drop_locked(dev);
+}
+
+}  // namespace
+
+namespace gbw {
+
+bool drop_kept_workspace(int dev) {
+  if (dev < 0 || dev >= kWorkDevices) return false;
+  std::lock_guard<std::mutex> lock(g_work.mu);
+  return drop_locked(dev);
+}
+
+cudaError_t device_malloc(void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  int dev = -1;
+  if (e == cudaErrorMemoryAllocation && cudaGetDevice(&dev) == cudaSuccess &&
+      drop_kept_workspace(dev)) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
+}  // namespace gbw
+
 namespace {
 
 size_t round_up256(size_t x) { return (x + 255) & ~size_t(255); }
+
+int ensure_for(const wave_ctx *c, DeviceBuf &b, size_t bytes) {
+  const int st = ensure(b, bytes, c->stream);
+  if (st != WAVE_ENOMEM || !drop_kept_workspace(c->device)) return st;
+  cudaGetLastError();
+  return ensure(b, bytes, c->stream);
+}
 
 int make_map(CUtensorMap *m, const void *base, const wave_ctx *c, int box_x,
              int box_y, CUtensorMapDataType dtype, int pitch, int esize) {
@@ -472,6 +541,7 @@ void wave_destroy(wave_ctx *c) {
   free_cpml(c);
   cudaFree(c->srec.p);
   cudaFree(c->d_nsrec);
+  if (c->counted) count_context(c->device, -1);
   delete c;
 }
 
@@ -515,6 +585,8 @@ static int alloc_context(wave_ctx *c) {
   const char *ev = std::getenv("GBWAVE_VARIANT");
   c->var = pick_variant(c->storage, ev ? std::atoi(ev) : 0);
   WAVE_TRY_CUDA(cudaGetDevice(&c->device));
+  count_context(c->device, 1);
+  c->counted = true;
   WAVE_TRY_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount,
                                        c->device));
   WAVE_TRY_CUDA(cudaStreamCreateWithFlags(&c->capture_stream,
@@ -524,7 +596,7 @@ static int alloc_context(wave_ctx *c) {
   const size_t off1 = round_up256(fbytes), offc = off1 + round_up256(fbytes);
   const size_t offd = offc + round_up256(bytes);
   const size_t offs = offd + round_up256(sizeof(StepDesc));
-  WAVE_TRY_CUDA(cudaMalloc(&c->base, offs + 256));
+  WAVE_TRY_CUDA(device_malloc(&c->base, offs + 256));
   char *base = static_cast<char *>(c->base);
   c->buf[0] = base;
   c->buf[1] = base + off1;
@@ -845,7 +917,7 @@ int propagate_begin(wave_ctx *c, const wave_shot *shot, int nsteps,
   const size_t o_start = take(nrec > 0 ? (size_t)(c->ntiles + 1) * 4 : 0);
   const size_t o_cnt = take(nrec > 0 ? (size_t)(c->ntiles + 1) * 4 : 0);
   const size_t o_tr = take(host_traces ? (size_t)nsteps * nrec * 4 : 0);
-  if ((s = ensure(c->tables, off, st))) return s;
+  if ((s = ensure_for(c, c->tables, off))) return s;
   char *tb = static_cast<char *>(c->tables.p);
   c->d_wavelet = reinterpret_cast<float *>(tb + o_w);
   c->d_rec = reinterpret_cast<int4 *>(tb + o_rec);
@@ -893,7 +965,7 @@ int propagate_begin(wave_ctx *c, const wave_shot *shot, int nsteps,
     // receivers inside the CPML shell are recorded from the shell values
     if (nrec > 0) {
       void *old = c->srec.p;
-      if ((s = ensure(c->srec, (size_t)nrec * sizeof(int4), st))) return s;
+      if ((s = ensure_for(c, c->srec, (size_t)nrec * sizeof(int4)))) return s;
       if (c->srec.p != old) drop_graphs(c);  // graphs hold the list's address
     }
     WAVE_TRY_CUDA(cudaMemsetAsync(c->d_nsrec, 0, sizeof(int), st));
@@ -1019,7 +1091,7 @@ int wave_get_field(const wave_ctx *c, int which, float *out) {
   // 16-bit storage: expand to FP32 with the field's scale.
   const size_t n = (size_t)c->nx * c->ny * c->nz;
   float *dst = out;
-  if (host_out) WAVE_TRY_CUDA(cudaMalloc((void **)&dst, n * 4));
+  if (host_out) WAVE_TRY_CUDA(device_malloc((void **)&dst, n * 4));
   if (c->storage == WAVE_STORAGE_BF16)
     launch_from_stored<__nv_bfloat16>(c, dst, src, field_slot(c, which));
   else
@@ -1055,7 +1127,7 @@ static int set_state_16(wave_ctx *c, const float *u, const float *u_prev,
   int status = WAVE_OK;
   for (int b = 0; b < 2 && status == WAVE_OK; ++b) {
     if (!is_device_ptr(src[b])) {
-      cudaError_t e = cudaMalloc((void **)&tmp[b], n * 4);
+      cudaError_t e = device_malloc((void **)&tmp[b], n * 4);
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(tmp[b], src[b], n * 4, cudaMemcpyHostToDevice, st);
       if (e != cudaSuccess) status = cuda_status(e);
@@ -1185,7 +1257,7 @@ int wave_set_cpml(wave_ctx *c, int npml, double R, double f_cps) {
     const size_t sl[3] = {2ull * npml * c->ny * c->nz, 2ull * npml * c->nz * c->nx,
                           2ull * npml * c->ny * c->nx};
     auto dalloc = [&](void **p, size_t bytes) -> int {
-      cudaError_t e = cudaMalloc(p, std::max<size_t>(bytes, 256));
+      cudaError_t e = device_malloc(p, std::max<size_t>(bytes, 256));
       if (e != cudaSuccess) return cuda_status(e);
       c->cpml_mem.push_back(*p);
       return WAVE_OK;
@@ -1213,7 +1285,7 @@ int wave_set_cpml(wave_ctx *c, int npml, double R, double f_cps) {
       cpml_axis_coefs(g, ax, hs[ax]);
     }
     cpml_plan_forms(c->cp);
-    if (!c->d_nsrec) WAVE_TRY_CUDA(cudaMalloc((void **)&c->d_nsrec, sizeof(int)));
+    if (!c->d_nsrec) WAVE_TRY_CUDA(device_malloc((void **)&c->d_nsrec, sizeof(int)));
     WAVE_TRY_CUDA(cudaMemset(c->d_nsrec, 0, sizeof(int)));
     c->cpml = true;
     if ((e = zero_cpml(c))) return e;
@@ -1387,19 +1459,59 @@ __global__ void grad_assemble_kernel(const double *gacc, const float *c,
   }
 }
 
-struct DevFree {  // frees the registered device buffers on scope exit
-  std::vector<void *> ptrs;
-  ~DevFree() {
-    for (void *p : ptrs) cudaFree(p);
+// A gradient call's device buffers: asked for one by one, then placed in one
+// block (KeptWork). Freed on scope exit, or kept after done().
+struct Workspace {
+  int dev;
+  void *block = nullptr;
+  size_t cap = 0, bytes = 0;
+  bool keep = false;
+  std::vector<std::pair<void **, size_t>> asked;
+
+  explicit Workspace(int d) : dev(d) {}
+  ~Workspace() {
+    if (!block) return;
+    if (keep) {
+      size_t all = 0, avail = 0;
+      std::lock_guard<std::mutex> lock(g_work.mu);
+      if (dev >= 0 && dev < kWorkDevices && !g_work.p[dev] && g_work.contexts[dev] > 0 &&
+          cudaMemGetInfo(&avail, &all) == cudaSuccess && cap <= all / 16) {
+        g_work.p[dev] = block;
+        g_work.cap[dev] = cap;
+        return;
+      }
+    }
+    cudaFree(block);
   }
   template <class T>
-  int alloc(T **p, size_t bytes) {
-    *p = nullptr;
-    cudaError_t e = cudaMalloc((void **)p, std::max<size_t>(bytes, 256));
-    if (e != cudaSuccess) return cuda_status(e);
-    ptrs.push_back(*p);
+  void ask(T **p, size_t n) {
+    asked.emplace_back((void **)p, bytes);
+    bytes += (std::max<size_t>(n, 1) + 511) & ~size_t(511);
+  }
+  int place() {
+    if (dev >= 0 && dev < kWorkDevices) {
+      std::lock_guard<std::mutex> lock(g_work.mu);
+      if (g_work.cap[dev] >= bytes) {
+        block = g_work.p[dev];
+        cap = g_work.cap[dev];
+        g_work.p[dev] = nullptr;
+        g_work.cap[dev] = 0;
+      } else {
+        drop_locked(dev);  // too small: this call's block is kept instead
+      }
+    }
+    if (!block) {
+      const cudaError_t e = device_malloc(&block, bytes);
+      if (e != cudaSuccess) {
+        block = nullptr;
+        return cuda_status(e);
+      }
+      cap = bytes;
+    }
+    for (auto &a : asked) *a.first = static_cast<char *>(block) + a.second;
     return WAVE_OK;
   }
+  void done() { keep = true; }
 };
 
 int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
@@ -1418,7 +1530,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   const size_t fb = fe * 4;
   const int ncp = (N + K - 1) / K;
   const size_t tn = (size_t)N * nrec;
-  DevFree mem;
+  Workspace mem(c->device);
   float *ckpt, *dbuf, *padj[2], *trd, *res, *inj, *wl, *ghi, *glo;
   double *gacc, *dmis;
   StepDesc *dadj, *dfwd;
@@ -1430,15 +1542,24 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   // its own fields, so the last segment's recompute can also run beside the
   // forward's last segment.
   const int nslot = ncp > 1 ? 2 : 1;
-  if ((e = mem.alloc(&ckpt, fb * 2 * ncp)) || (e = mem.alloc(&dbuf, fb * K * nslot)) ||
-      (e = mem.alloc(&padj[0], fb)) || (e = mem.alloc(&padj[1], fb)) ||
-      (e = mem.alloc(&trd, tn * 4)) || (e = mem.alloc(&res, tn * 4)) ||
-      (e = mem.alloc(&inj, (tn + nrec) * 4)) || (e = mem.alloc(&wl, (size_t)N * 4)) ||
-      (e = mem.alloc(&gacc, fe * 8)) || (e = mem.alloc(&dmis, 8)) ||
-      (e = mem.alloc(&ghi, fb)) || (e = mem.alloc(&glo, fb)) ||
-      (e = mem.alloc(&dadj, sizeof(StepDesc))) ||
-      (e = mem.alloc(&dfwd, sizeof(StepDesc))))
-    return e;
+  mem.ask(&ckpt, fb * 2 * ncp);
+  mem.ask(&dbuf, fb * K * nslot);
+  mem.ask(&padj[0], fb);
+  mem.ask(&padj[1], fb);
+  mem.ask(&trd, tn * 4);
+  mem.ask(&res, tn * 4);
+  mem.ask(&inj, (tn + nrec) * 4);
+  mem.ask(&wl, (size_t)N * 4);
+  mem.ask(&gacc, fe * 8);
+  mem.ask(&dmis, 8);
+  mem.ask(&ghi, fb);
+  mem.ask(&glo, fb);
+  mem.ask(&dadj, sizeof(StepDesc));
+  mem.ask(&dfwd, sizeof(StepDesc));
+  const size_t ne = (size_t)c->nx * c->ny * c->nz;
+  const bool host_grad = !is_device_ptr(grad);
+  float *gout = grad;
+  if (host_grad) mem.ask(&gout, ne * 4);
   // With the CPML layer: the memory variables psi, zeta (per axis) are saved
   // with each checkpoint, the recompute steps the saved copies in place, and
   // the adjoint carries its nu, mu slabs.
@@ -1449,11 +1570,13 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
     sl[0] = 2ull * cg.npml * c->ny * c->nz;
     sl[1] = 2ull * cg.npml * c->nz * c->nx;
     sl[2] = 2ull * cg.npml * c->ny * c->nx;
-    if ((e = mem.alloc(&ckpt_l, (sl[0] + sl[1] + sl[2]) * 2 * 4 * ncp))) return e;
-    for (int ax = 0; ax < 3; ++ax)
-      if ((e = mem.alloc(&nus[ax], sl[ax] * 4)) || (e = mem.alloc(&mus[ax], sl[ax] * 4)))
-        return e;
+    mem.ask(&ckpt_l, (sl[0] + sl[1] + sl[2]) * 2 * 4 * ncp);
+    for (int ax = 0; ax < 3; ++ax) {
+      mem.ask(&nus[ax], sl[ax] * 4);
+      mem.ask(&mus[ax], sl[ax] * 4);
+    }
   }
+  if ((e = mem.place())) return e;
   // the layer slabs held by a segment's checkpoint (per axis psi, then zeta)
   auto layer_of = [&](int sgm) {
     CpmlPlan pl = c->cp;
@@ -1680,10 +1803,6 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   WAVE_TRY_CUDA(cudaGetLastError());
 
   // Gradient, traces, misfit.
-  const size_t ne = (size_t)c->nx * c->ny * c->nz;
-  float *gout = grad;
-  const bool host_grad = !is_device_ptr(grad);
-  if (host_grad && (e = mem.alloc(&gout, ne * 4))) return e;
   grad_assemble_kernel<<<c->sms * 4, 256, 0, st>>>(
       gacc, c->c, gout, c->nx, c->px, (long long)c->ny * c->nz, c->dt * c->dt);
   WAVE_TRY_CUDA(cudaGetLastError());
@@ -1698,6 +1817,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   WAVE_TRY_CUDA(cudaMemcpyAsync(&errs[0], &dfwd->error, 4, cudaMemcpyDeviceToHost, st));
   WAVE_TRY_CUDA(cudaMemcpyAsync(&errs[1], &dadj->error, 4, cudaMemcpyDeviceToHost, st));
   WAVE_TRY_CUDA(cudaStreamSynchronize(st));
+  mem.done();  // every kernel that uses the workspace has finished
   if (misfit && !data_is_resid) *misfit = hm;
   // errors of the forward run (a timeout, or NaN in its traces), read before
   // the reset clears them
