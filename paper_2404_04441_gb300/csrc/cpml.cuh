@@ -936,6 +936,28 @@ struct CpmlPass {
   float *nus[3], *mus[3];
 };
 
+// The shell receivers' row of the step before this pass's: u^n is that step's
+// field with the layer's terms, and nothing writes it during this step, so the
+// row rides in blocks beside the lines instead of in a launch of its own after
+// them (3 us a step; the last step's row is recorded at the call's end).
+constexpr int kCpmlRecClusters = 8;
+
+template <class T>
+__device__ __forceinline__ void cpml_record_previous(const CpmlGeom &g, const CpmlPass &a,
+                                                     int first, int step) {
+  const long long n = a.d->n + a.koff;
+  const int nr = *a.nsrec;
+  if (n == 0 || nr == 0) return;
+  CpmlScale<T> sc;
+  sc.init(a.d, a.koff);
+  const T *u = static_cast<const T *>(a.u);
+  float *row = a.d->traces + (size_t)(n - 1) * a.d->nrec;
+  for (int r = first; r < nr; r += step) {
+    const int4 e = a.srec[r];
+    row[e.w] = cpml_get(u + ((size_t)e.z * g.ny + e.y) * g.pxu + e.x, sc.su);
+  }
+}
+
 // Release and acquire over the cluster: global writes before it are visible
 // to the cluster's reads after it.
 __device__ __forceinline__ void cpml_cluster_sync() {
@@ -948,6 +970,11 @@ __device__ __forceinline__ void cpml_cluster_sync() {
 template <int NPML_, class T, bool kStoreD>
 struct CpmlForward {
   static constexpr int NPML = NPML_;
+  static constexpr bool kRecords = !kStoreD;
+  __device__ static __forceinline__ void record_previous(const CpmlGeom &g, const CpmlPass &a,
+                                                         int first, int step) {
+    cpml_record_previous<T>(g, a, first, step);
+  }
   template <int AX, int SIDE, class P>
   __device__ static __forceinline__ void line(const CpmlGeom &g, const P &pf, const CpmlPass &a,
                                               int p, int q, const CpmlScale<T> &sc) {
@@ -966,6 +993,9 @@ struct CpmlForward {
 template <int NPML_>
 struct CpmlAdjoint {
   static constexpr int NPML = NPML_;
+  static constexpr bool kRecords = false;
+  __device__ static __forceinline__ void record_previous(const CpmlGeom &, const CpmlPass &, int,
+                                                         int) {}
   template <int AX, int SIDE, class P>
   __device__ static __forceinline__ void line(const CpmlGeom &g, const P &pf, const CpmlPass &a,
                                               int p, int q, const CpmlScale<float> &) {
@@ -1002,11 +1032,16 @@ __global__ void __cluster_dims__(kCpmlCluster, 1, 1) __launch_bounds__(kCpmlThre
     cpml_lines_kernel(const __grid_constant__ CpmlGeom g, const __grid_constant__ CpmlTiles t,
                       const __grid_constant__ CpmlProf<OP::NPML> pf,
                       const __grid_constant__ CpmlPass a) {
-  cpml_lines<OP>(g, t, pf, a, blockIdx.x / kCpmlCluster);
+  const int blk = blockIdx.x / kCpmlCluster;
+  if (OP::kRecords && blk >= t.start[7])
+    OP::record_previous(g, a, (blockIdx.x - t.start[7] * kCpmlCluster) * kCpmlThreads + threadIdx.x,
+                        kCpmlRecClusters * kCpmlLines);
+  else
+    cpml_lines<OP>(g, t, pf, a, blk);
 }
 
 // Receivers within w of a face: {x, y, z, receiver id}, recorded from the
-// field after the three axis passes (16-bit: the stored value times its
+// field after the step's layer terms (16-bit: the stored value times its
 // scale).
 template <class T>
 __global__ void cpml_record_kernel(CpmlGeom g, const T *__restrict__ unext,
@@ -1052,9 +1087,13 @@ inline void cpml_plan_forms(CpmlPlan &p) {
 
 // Launches, enqueued on st (layer.cu): one forward step's layer terms and
 // shell receivers (store_d: also into D, no receivers), one adjoint step's.
-// a.koff and the descriptor give the step.
+// a.koff and the descriptor give the step. Where every axis is unrolled a
+// step records the receivers of the step before (cpml_record_previous), and
+// cpml_record_last those of the last step once the descriptor is past it.
 void cpml_forward(int storage, bool store_d, const CpmlPlan &p, const CpmlPass &a, int sms,
                   cudaStream_t st);
+void cpml_record_last(int storage, const CpmlPlan &p, const CpmlPass &a, int sms,
+                      cudaStream_t st);
 void cpml_adjoint(const CpmlPlan &p, const CpmlPass &a, cudaStream_t st);
 
 // The unrolled line ends on tiles t of the plan (layer_lines.cuh, compiled

@@ -22,6 +22,12 @@ void walk_adjoint(const CpmlPlan &p, const CpmlPass &a, cudaStream_t st) {
       a.mus[AX]);
 }
 
+template <class T>
+void record(const CpmlPlan &p, const CpmlPass &a, int sms, cudaStream_t st) {
+  cpml_record_kernel<T><<<sms, 256, 0, st>>>(p.g, static_cast<const T *>(a.unext), a.d, a.srec,
+                                             a.nsrec, a.koff);
+}
+
 template <class T, bool kD>
 void forward(const CpmlPlan &p, const CpmlPass &a, int sms, cudaStream_t st) {
   if (p.axes == 7) cpml_launch_lines<T, kD>(p, p.all, a, st);
@@ -35,9 +41,7 @@ void forward(const CpmlPlan &p, const CpmlPass &a, int sms, cudaStream_t st) {
     else
       walk<2, T, kD>(p, a, st);
   }
-  if constexpr (!kD)
-    cpml_record_kernel<T><<<sms, 256, 0, st>>>(p.g, static_cast<const T *>(a.unext), a.d, a.srec,
-                                               a.nsrec, a.koff);
+  if (!kD && p.axes != 7) record<T>(p, a, sms, st);
 }
 
 template <int AX, class T>
@@ -107,6 +111,17 @@ void cpml_forward(int storage, bool store_d, const CpmlPlan &p, const CpmlPass &
     forward<float, true>(p, a, sms, st);
   else
     forward<float, false>(p, a, sms, st);
+}
+
+void cpml_record_last(int storage, const CpmlPlan &p, const CpmlPass &a, int sms,
+                      cudaStream_t st) {
+  if (p.axes != 7) return;
+  if (storage == WAVE_STORAGE_BF16)
+    record<__nv_bfloat16>(p, a, sms, st);
+  else if (storage == WAVE_STORAGE_F16)
+    record<__half>(p, a, sms, st);
+  else
+    record<float>(p, a, sms, st);
 }
 
 void cpml_adjoint(const CpmlPlan &p, const CpmlPass &a, cudaStream_t st) {

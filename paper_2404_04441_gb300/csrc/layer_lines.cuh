@@ -64,7 +64,8 @@ void cpml_launch(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a, cudaS
       pf.b[f >> 1][f & 1][j] = p.prof.b[f >> 1][f & 1][j];
       pf.a[f >> 1][f & 1][j] = p.prof.a[f >> 1][f & 1][j];
     }
-  cpml_lines_kernel<OP><<<t.start[7] * kCpmlCluster, kCpmlThreads, 0, st>>>(p.g, t, pf, a);
+  const int clusters = t.start[7] + (OP::kRecords && t.all ? kCpmlRecClusters : 0);
+  cpml_lines_kernel<OP><<<clusters * kCpmlCluster, kCpmlThreads, 0, st>>>(p.g, t, pf, a);
 }
 
 template <class T, bool kStoreD>

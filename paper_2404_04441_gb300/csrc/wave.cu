@@ -400,6 +400,10 @@ int run_steps(wave_ctx *c, int nsteps) {
     advance_kernel<<<1, 1, 0, c->stream>>>(c->d_desc, rem);
     c->cur = cur;
   }
+  // the last step's shell receivers: the descriptor's counter is past it
+  if (c->cpml && nsteps > 0 && c->host_desc.nrec > 0)
+    cpml_record_last(c->storage, c->cp,
+                     layer_pass(c, c->buf[c->cur ^ 1], c->buf[c->cur], -1), c->sms, c->stream);
   WAVE_TRY_CUDA(cudaGetLastError());
   c->step += nsteps;
   if (nsteps > 0) c->at_rest = false;
