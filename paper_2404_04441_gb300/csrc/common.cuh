@@ -532,7 +532,7 @@ int plan_candidate_chunks(int nz, const PlanCandidate &pc, int *out) {
   }
   int rest = nz - pc.tail * pc.b;
   const int full = rest / pc.a;
-  if (full + (rest % pc.a > 0) + pc.tail > kMaxLayers) return 0;
+  if (full + (rest % pc.a > 0) + pc.tail > kPlanLayers) return 0;
   while (rest >= pc.a) {
     out[n++] = pc.a;
     rest -= pc.a;
@@ -542,23 +542,23 @@ int plan_candidate_chunks(int nz, const PlanCandidate &pc, int *out) {
   return n;
 }
 
-// Split nz into at most kMaxLayers z layers, chosen by layer_makespan: a
+// Split nz into at most kPlanLayers z layers, chosen by layer_makespan: a
 // cheap score (work plus waves) ranks all candidates; every uniform split
 // and the best-ranked others (among the 48 best scores) are simulated, and
 // the first plan with the smallest makespan wins. Writes the plan to out and
 // returns its layer count. Fixed storage only (no allocation).
 int plan_layers(int nz, long long ntiles, long long slots, double preroll,
-                int out[kMaxLayers]) {
+                int out[kPlanLayers]) {
   constexpr int kTop = 48;
   static const int kTail[6] = {8, 16, 24, 32, 48, 64};
-  const int nuni = std::min(nz, kMaxLayers);
+  const int nuni = std::min(nz, kPlanLayers);
   // the kTop best (score, index) pairs, ascending
   double tscore[kTop] = {};
   int tidx[kTop] = {};
   PlanCandidate tcand[kTop] = {};
   int ntop = 0;
   int idx = 0;
-  int ch[kMaxLayers];
+  int ch[kPlanLayers];
   auto consider = [&](const PlanCandidate &pc) {
     const int n = plan_candidate_chunks(nz, pc, ch);
     if (n == 0) return;
@@ -605,9 +605,32 @@ int plan_layers(int nz, long long ntiles, long long slots, double preroll,
   return best_n;
 }
 
+// Halves a plan's layers (in place; room for kMaxLayers) while each half keeps
+// two planes and the launch at most `limit` CTAs. On a grid of a few tiles the
+// planner's 16 layers leave the chip idle: a CTA's planes come one after
+// another at their latency (about 1000 cycles each) whoever else runs, and the
+// starts of more CTAs (2600 cycles to the first plane, 8 more planes of u from
+// L2) overlap. FP32, 3 CTAs an SM, us a step: 64^3 4.31 -> 3.52, 32 x 16 x 512
+// 14.9 -> 5.9, 96 x 64 x 96 5.79 -> 4.94, 64 x 64 x 200 8.2 -> 6.3 (4 CTAs an
+// SM: 128 x 64 x 64 4.91 -> 5.04; layers of one plane: 64^3 3.96). 16-bit, 2 an
+// SM: 64^3 5.66 -> 4.77, 48 x 90 x 60 5.59 -> 5.40 (3: 128 x 96 x 100 7.7 ->
+// 10.2). Returns the new layer count.
+int split_layers(int *ch, int n, long long ntiles, long long limit) {
+  while (2 * n <= kMaxLayers && 2 * n * ntiles <= limit &&
+         *std::min_element(ch, ch + n) >= 4) {
+    for (int i = n - 1; i >= 0; --i) {
+      const int c = ch[i];
+      ch[2 * i] = (c + 1) / 2;
+      ch[2 * i + 1] = c / 2;
+    }
+    n *= 2;
+  }
+  return n;
+}
+
 std::vector<int> plan_layers(int nz, long long ntiles, long long slots,
                              double preroll = 4.0) {
-  int out[kMaxLayers];
+  int out[kPlanLayers];
   const int n = plan_layers(nz, ntiles, slots, preroll, out);
   return std::vector<int>(out, out + n);
 }

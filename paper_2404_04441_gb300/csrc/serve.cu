@@ -126,7 +126,7 @@ size_t layer_bytes(const wave_request &r) {
 // Device bytes of a request once resident (the budget unit).
 // z layers of a batched shot: at most kLayerPlanes planes each, equal sizes.
 int request_layers(int nz) {
-  return std::min(kMaxLayers, std::max(1, (nz + kLayerPlanes - 1) / kLayerPlanes));
+  return std::min(kPlanLayers, std::max(1, (nz + kLayerPlanes - 1) / kLayerPlanes));
 }
 
 // CTAs one batched step launches for the request.

@@ -65,7 +65,8 @@ struct StepDesc {
   unsigned maxbits[4];
 };
 
-constexpr int kMaxLayers = 16;
+constexpr int kPlanLayers = 16;  // z layers of a plan (plan_layers)
+constexpr int kMaxLayers = 64;   // z layers of a launch (split_layers)
 
 // Extra work of a sweep (template bit mask), used by the adjoint gradient:
 constexpr int kModeStoreD = 1;   // write D = v^2 dt^2 (L u) + source to a.dout

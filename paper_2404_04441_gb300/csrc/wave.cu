@@ -628,8 +628,10 @@ static int setup_launch(wave_ctx *c) {
   int layers[kMaxLayers];
   double preroll = c->storage == WAVE_STORAGE_F32 ? 4.0 : 8.0;
   if (const char *pr = std::getenv("GBWAVE_PREROLL")) preroll = std::atof(pr);
-  const int nl = plan_layers(c->nz, (long long)c->ntiles,
-                             (long long)c->sms * c->ctas_per_sm, preroll, layers);
+  int nl = plan_layers(c->nz, (long long)c->ntiles, (long long)c->sms * c->ctas_per_sm,
+                       preroll, layers);
+  nl = split_layers(layers, nl, c->ntiles,
+                    (c->storage == WAVE_STORAGE_F32 ? 3ll : 2ll) * c->sms);
   c->zchunk = *std::max_element(layers, layers + nl);
   c->grid = dim3(ntx, nty, (unsigned)nl);
   if (c->grid.y > 65535) return WAVE_EINVAL;
@@ -1371,8 +1373,10 @@ struct GradStreams {
 // shorter layers fill the CTA places better).
 dim3 plan_mode(const wave_ctx *c, double preroll, SweepArgs &a) {
   int layers[kMaxLayers];
-  const int nl = plan_layers(c->nz, (long long)c->ntiles,
-                             (long long)c->sms * c->ctas_per_sm, preroll, layers);
+  int nl = plan_layers(c->nz, (long long)c->ntiles, (long long)c->sms * c->ctas_per_sm,
+                       preroll, layers);
+  nl = split_layers(layers, nl, c->ntiles,
+                    (c->storage == WAVE_STORAGE_F32 ? 3ll : 2ll) * c->sms);
   set_layers(a, layers, nl);
   return dim3(c->grid.x, c->grid.y, (unsigned)nl);
 }
@@ -2060,8 +2064,8 @@ extern "C" int wave_propagate_noalloc(const wave_grid *g, const wave_spacing *h,
   }
   if ((st = noalloc_map(&vmap, velocity, nx, ny, nz, C::TX, C::TY))) return st;
   int layers[kMaxLayers];
-  const int nl = plan_layers(nz, (long long)ntiles,
-                             (long long)nd->sms * nd->ctas_per_sm, 4.0, layers);
+  int nl = plan_layers(nz, (long long)ntiles, (long long)nd->sms * nd->ctas_per_sm, 4.0, layers);
+  nl = split_layers(layers, nl, (long long)ntiles, 2ll * nd->sms);
   const dim3 grid(ntx, nty, (unsigned)nl);
   if (grid.y > 65535) return WAVE_EINVAL;
   SweepArgs a{};

@@ -1,6 +1,6 @@
 """The sweep's z layers at the sizes where its prologue and ring can go wrong:
-layers of one to a few planes (fewer stages than the ring has slots), grids
-whose layers start at, above and below a receiver plane, receivers at every
+layers of one to a few planes (fewer stages than the ring has slots), grids of
+a few tiles, whose plans are split into up to 64 layers, grids whose layers start at, above and below a receiver plane, receivers at every
 depth and repeated, against the FP64 oracle.
 
 FP32: relative L2 <= 1e-5, the bar of the parity tests. FP16: each step rounds
@@ -18,7 +18,8 @@ import workloads as wl
 pytestmark = pytest.mark.gpu
 
 CASES = [((37, 21, nz), 0) for nz in (1, 2, 3, 4, 5, 8, 13, 16, 17, 33, 63)] + \
-        [((72, 35, nz), 2) for nz in (1, 3, 4, 5, 9, 17, 40)]
+        [((72, 35, nz), 2) for nz in (1, 3, 4, 5, 9, 17, 40)] + \
+        [((37, 21, nz), 0) for nz in (64, 67, 130, 260)] + [((72, 35, nz), 2) for nz in (64, 131)]
 
 
 def rel_l2(a, b):
