@@ -1028,7 +1028,7 @@ __device__ __forceinline__ void cpml_lines(const CpmlGeom &g, const CpmlTiles &t
 }
 
 template <class OP>
-__global__ void __cluster_dims__(kCpmlCluster, 1, 1) __launch_bounds__(kCpmlThreads, cpml_ctas(OP::NPML))
+__global__ void __launch_bounds__(kCpmlThreads, cpml_ctas(OP::NPML))
     cpml_lines_kernel(const __grid_constant__ CpmlGeom g, const __grid_constant__ CpmlTiles t,
                       const __grid_constant__ CpmlProf<OP::NPML> pf,
                       const __grid_constant__ CpmlPass a) {
@@ -1065,9 +1065,19 @@ struct CpmlPlan {
   CpmlGeom g;
   int axes;     // bit a: axis a takes the unrolled line ends
   int variant;  // which width (cpml_variant)
+  // All three unrolled, but one launch per axis (kCpmlByAxis line ends or more).
+  bool by_axis;
   CpmlProf<kCpmlMaxCap> prof;
   CpmlTiles all, one[3];  // every axis at once; single axes
 };
+
+// Line ends from which the axes take a launch each, without clusters: the
+// launches' ends no longer count, and the cluster launch fills the chip a
+// little less evenly. 16 cells, us a step in one launch and by axis: FP32 1024 x
+// 1024 x 512 (4.2 M) 1736 and 1709, FP16 1319 and 1292, 512^3 (1.6 M) 514 and
+// 508, 512 x 512 x 256 (1.0 M) 288 and 292; BF16 513 x 511 x 300 (1.1 M) 308 and
+// 313.
+constexpr long long kCpmlByAxis = 1500000;
 
 // Takes the plan's form on each axis from the grid and the layer's width
 // (g.npml set), and its tiles.
@@ -1081,6 +1091,8 @@ inline void cpml_plan_forms(CpmlPlan &p) {
   for (int ax = 0; ax < 3; ++ax)
     if (cpml_seg_fits(g.npml, n[ax], fstep[ax], sstep[ax])) p.axes |= 1 << ax;
   p.variant = cpml_variant(g.npml);
+  p.by_axis = p.axes == 7 && 2 * ((long long)g.ny * g.nz + (long long)g.nx * g.nz +
+                                  (long long)g.nx * g.ny) >= kCpmlByAxis;
   p.all = cpml_tiles(g.nx, g.ny, g.nz, g.w, -1);
   for (int ax = 0; ax < 3; ++ax) p.one[ax] = cpml_tiles(g.nx, g.ny, g.nz, g.w, ax);
 }
@@ -1097,9 +1109,10 @@ void cpml_record_last(int storage, const CpmlPlan &p, const CpmlPass &a, int sms
 void cpml_adjoint(const CpmlPlan &p, const CpmlPass &a, cudaStream_t st);
 
 // The unrolled line ends on tiles t of the plan (layer_lines.cuh, compiled
-// once per storage type, and for the gradient).
+// once per storage type, and for the gradient); record: with the shell
+// receivers of the step before.
 template <class T, bool kStoreD>
-void cpml_launch_lines(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a,
+void cpml_launch_lines(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a, bool record,
                        cudaStream_t st);
 void cpml_launch_adjoint_lines(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a,
                                cudaStream_t st);

@@ -30,10 +30,11 @@ void record(const CpmlPlan &p, const CpmlPass &a, int sms, cudaStream_t st) {
 
 template <class T, bool kD>
 void forward(const CpmlPlan &p, const CpmlPass &a, int sms, cudaStream_t st) {
-  if (p.axes == 7) cpml_launch_lines<T, kD>(p, p.all, a, st);
-  for (int ax = 0; ax < 3 && p.axes != 7; ++ax) {
+  const bool all = p.axes == 7 && !p.by_axis;
+  if (all) cpml_launch_lines<T, kD>(p, p.all, a, true, st);
+  for (int ax = 0; ax < 3 && !all; ++ax) {
     if ((p.axes >> ax) & 1)
-      cpml_launch_lines<T, kD>(p, p.one[ax], a, st);
+      cpml_launch_lines<T, kD>(p, p.one[ax], a, p.axes == 7 && ax == 0, st);
     else if (ax == 0)
       walk<0, T, kD>(p, a, st);
     else if (ax == 1)
@@ -125,8 +126,9 @@ void cpml_record_last(int storage, const CpmlPlan &p, const CpmlPass &a, int sms
 }
 
 void cpml_adjoint(const CpmlPlan &p, const CpmlPass &a, cudaStream_t st) {
-  if (p.axes == 7) cpml_launch_adjoint_lines(p, p.all, a, st);
-  for (int ax = 0; ax < 3 && p.axes != 7; ++ax) {
+  const bool all = p.axes == 7 && !p.by_axis;
+  if (all) cpml_launch_adjoint_lines(p, p.all, a, st);
+  for (int ax = 0; ax < 3 && !all; ++ax) {
     if ((p.axes >> ax) & 1)
       cpml_launch_adjoint_lines(p, p.one[ax], a, st);
     else if (ax == 0)

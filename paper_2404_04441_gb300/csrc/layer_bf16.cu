@@ -4,7 +4,7 @@
 namespace gbw {
 
 template void cpml_launch_lines<__nv_bfloat16, false>(const CpmlPlan &, const CpmlTiles &, const CpmlPass &,
-                                           cudaStream_t);
+                                           bool, cudaStream_t);
 template void cpml_launch_batched_lines<__nv_bfloat16>(int, int, const CpmlBatchShot *, int, int, long long,
                                             cudaStream_t);
 

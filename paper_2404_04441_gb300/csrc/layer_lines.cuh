@@ -38,7 +38,7 @@ __device__ __forceinline__ bool cpml_batch_pass(const CpmlBatchShot &sh, long lo
 // the single-grid kernel takes it from its parameters). A cluster's CTAs
 // belong to one shot: its first block is a multiple of the cluster.
 template <class OP>
-__global__ void __cluster_dims__(kCpmlCluster, 1, 1) __launch_bounds__(kCpmlThreads, cpml_ctas(OP::NPML))
+__global__ void __launch_bounds__(kCpmlThreads, cpml_ctas(OP::NPML))
     cpml_lines_batched_kernel(const CpmlBatchShot *__restrict__ shots, int nshots, long long k,
                               int ax) {
   const int which = ax < 0 ? 0 : ax;
@@ -56,26 +56,44 @@ __global__ void __cluster_dims__(kCpmlCluster, 1, 1) __launch_bounds__(kCpmlThre
                  (int)(blockIdx.x - sh.blk_begin[which]) / kCpmlCluster);
 }
 
+// Launch of `blocks` CTAs, in clusters where several axes' lines meet (one
+// axis's lines need no barrier).
+template <class K, class... Args>
+void cpml_launch_grid(K kernel, int blocks, bool clusters, cudaStream_t st, const Args &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(kCpmlThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kCpmlCluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = clusters ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <class OP>
-void cpml_launch(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a, cudaStream_t st) {
+void cpml_launch(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a, bool record,
+                 cudaStream_t st) {
   CpmlProf<OP::NPML> pf;
   for (int f = 0; f < 6; ++f)
     for (int j = 0; j < OP::NPML; ++j) {
       pf.b[f >> 1][f & 1][j] = p.prof.b[f >> 1][f & 1][j];
       pf.a[f >> 1][f & 1][j] = p.prof.a[f >> 1][f & 1][j];
     }
-  const int clusters = t.start[7] + (OP::kRecords && t.all ? kCpmlRecClusters : 0);
-  cpml_lines_kernel<OP><<<clusters * kCpmlCluster, kCpmlThreads, 0, st>>>(p.g, t, pf, a);
+  const int clusters = t.start[7] + (OP::kRecords && record ? kCpmlRecClusters : 0);
+  cpml_launch_grid(cpml_lines_kernel<OP>, clusters * kCpmlCluster, t.all, st, p.g, t, pf, a);
 }
 
 template <class T, bool kStoreD>
-void cpml_launch_lines(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a,
+void cpml_launch_lines(const CpmlPlan &p, const CpmlTiles &t, const CpmlPass &a, bool record,
                        cudaStream_t st) {
   switch (p.variant) {
-    case 0: return cpml_launch<CpmlForward<8, T, kStoreD>>(p, t, a, st);
-    case 1: return cpml_launch<CpmlForward<10, T, kStoreD>>(p, t, a, st);
-    case 2: return cpml_launch<CpmlForward<16, T, kStoreD>>(p, t, a, st);
-    default: return cpml_launch<CpmlForward<20, T, kStoreD>>(p, t, a, st);
+    case 0: return cpml_launch<CpmlForward<8, T, kStoreD>>(p, t, a, record, st);
+    case 1: return cpml_launch<CpmlForward<10, T, kStoreD>>(p, t, a, record, st);
+    case 2: return cpml_launch<CpmlForward<16, T, kStoreD>>(p, t, a, record, st);
+    default: return cpml_launch<CpmlForward<20, T, kStoreD>>(p, t, a, record, st);
   }
 }
 
@@ -84,20 +102,20 @@ void cpml_launch_batched_lines(int variant, int ax, const CpmlBatchShot *shots, 
                                long long k, cudaStream_t st) {
   switch (variant) {
     case 0:
-      cpml_lines_batched_kernel<CpmlForward<8, T, false>>
-          <<<blocks, kCpmlThreads, 0, st>>>(shots, n, k, ax);
+      cpml_launch_grid(cpml_lines_batched_kernel<CpmlForward<8, T, false>>, blocks, ax < 0, st,
+                       shots, n, k, ax);
       return;
     case 1:
-      cpml_lines_batched_kernel<CpmlForward<10, T, false>>
-          <<<blocks, kCpmlThreads, 0, st>>>(shots, n, k, ax);
+      cpml_launch_grid(cpml_lines_batched_kernel<CpmlForward<10, T, false>>, blocks, ax < 0, st,
+                       shots, n, k, ax);
       return;
     case 2:
-      cpml_lines_batched_kernel<CpmlForward<16, T, false>>
-          <<<blocks, kCpmlThreads, 0, st>>>(shots, n, k, ax);
+      cpml_launch_grid(cpml_lines_batched_kernel<CpmlForward<16, T, false>>, blocks, ax < 0, st,
+                       shots, n, k, ax);
       return;
     default:
-      cpml_lines_batched_kernel<CpmlForward<20, T, false>>
-          <<<blocks, kCpmlThreads, 0, st>>>(shots, n, k, ax);
+      cpml_launch_grid(cpml_lines_batched_kernel<CpmlForward<20, T, false>>, blocks, ax < 0, st,
+                       shots, n, k, ax);
   }
 }
 
