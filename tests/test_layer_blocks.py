@@ -17,7 +17,7 @@ GRIDS = [(10, 10, 10, 1), (11, 13, 10, 1), (24, 24, 24, 8), (25, 31, 24, 8), (28
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def walker(tmp_path_factory):
     nvcc = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "bin", "nvcc")
     if not os.path.exists(nvcc):
         nvcc = shutil.which("nvcc")
@@ -31,7 +31,7 @@ def checker(tmp_path_factory):
 
 
 @pytest.mark.parametrize("grid", GRIDS)
-def test_blocks_cover_the_layer_in_order(checker, grid):
-    out = subprocess.run([checker], input="%d %d %d %d\n" % grid, capture_output=True, text=True,
+def test_blocks_cover_the_layer_in_order(walker, grid):
+    out = subprocess.run([walker], input="%d %d %d %d\n" % grid, capture_output=True, text=True,
                          check=True).stdout
     assert out.strip() == "ok"
