@@ -541,8 +541,8 @@ __global__ void __launch_bounds__(128)
 // What bounds it: on small grids the launches and two memory latencies a
 // line (u^n, psi and zeta; then C and u^{n+1}), on large ones the traffic of
 // lines that every array is read along. Against one launch per axis (line
-// walks at 10 cells, unrolled at 16), a whole step took 31 us instead of 56
-// at 150 x 141 x 133 with 10 cells, 102 instead of 104 at 320 x 256 x 192 in
+// walks at 10 cells, unrolled at 16), with the sweep of that time, a whole step
+// took 31 us instead of 56 at 150 x 141 x 133 with 10 cells (25 now), 102 instead of 104 at 320 x 256 x 192 in
 // FP16 and 291 instead of 296 at 512 x 512 x 256 with 16; the gradient through
 // autograd at 160 x 144 x 128 x 100 steps 18.0 ms instead of 20.0. CTAs of 256
 // threads without clusters took 7 % longer at 320 x 256 x 192, 4 CTAs an SM
