@@ -265,11 +265,13 @@ int wave_get_launch_info(const wave_ctx *ctx, int *tile_x, int *tile_y,
                          int *z_chunk, int *grid_ctas, int *ctas_per_sm);
 
 /*
- * Diagnostic of the bounded device wait used by every kernel of this
- * library: launches one thread that waits on a shared-memory barrier nothing
- * arrives on, with a limit of limit_ns nanoseconds (clamped to 1 ms .. 10 s).
- * Synchronizes the stream. Returns WAVE_ETIMEOUT when the wait gave up as
- * designed, WAVE_ECUDA if it reported completion or a CUDA call failed.
+ * Diagnostic of the bounded device waits used by every kernel of this
+ * library: launches blocks that wait on shared-memory barriers nothing
+ * arrives on, with a limit of limit_ns nanoseconds (clamped to 1 ms .. 10 s):
+ * one alone, and the sweeps' ring of stages with each stage of 1 to 10 lost.
+ * Synchronizes the stream. Returns WAVE_ETIMEOUT when every wait gave up and
+ * every loss was seen as designed, WAVE_ECUDA if one was reported as complete
+ * or a CUDA call failed.
  * No counterpart in the paper (failure detection of this library).
  */
 int wave_selftest_wait(int64_t limit_ns, void *stream);

@@ -96,6 +96,33 @@ __device__ __forceinline__ void mbar_wait_or_flag(uint32_t bar, uint32_t parity,
   *failed = 1;
 }
 
+// The wait of a CTA's ring for its stage s: every thread waits by itself, then
+// one plain barrier. A stage that did not land is looked for every kRingLook
+// stages (a barrier that carries a verdict costs more than a plain one) and,
+// since the last stages need not be looked at, once more after the loop
+// (ring_failed): true if this or an earlier stage gave up. Until then a CTA
+// computes from what its slots hold; what it stores is void with the error.
+constexpr int kRingLook = 3;
+
+__device__ __forceinline__ bool ring_failed(volatile int *failed) {
+  return __builtin_expect(*failed, 0);
+}
+
+__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, uint64_t limit_ns,
+                                          volatile int *failed, bool look) {
+  mbar_wait_or_flag(bar, parity, limit_ns, failed);
+  __syncthreads();
+  return look && ring_failed(failed);
+}
+
+// Waits, each within limit_ns, for the stages [first, end) of a ring of NB
+// barriers, so that no TMA write lands in shared memory after the CTA exits.
+template <int NB>
+__device__ __forceinline__ void ring_drain(uint64_t *bars, int first, int end,
+                                           uint64_t limit_ns) {
+  for (int t = first; t < end; ++t) mbar_wait_bounded(&bars[t % NB], (t / NB) & 1, limit_ns);
+}
+
 // 3D tiled TMA load of one box into shared memory; completion is signalled
 // on the barrier as transaction bytes. Coordinates are element indices
 // (x innermost) and may lie outside the tensor: those elements read as zero.

@@ -516,7 +516,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       q[v][p] = E::load4(su + p * C::U_SLOT + (ty * C::VY + v + kR) * C::UW + col);
     if (p == kR - 1) {
       __syncthreads();
-      if (*failed) goto wait_failed;
+      if (ring_failed(failed)) goto wait_failed;
       if (tid == 0)
         for (int t = C::SU; t < 2 * kR + C::PF && t < NS; ++t) issue(t);
     }
@@ -529,12 +529,11 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       if (s >= NS) break;
       // One barrier per plane: stage s has landed for every thread, and
       // every thread is done with plane s-1, whose slots the next issue may
-      // overwrite. A wait that gave up is looked for every third plane (a
-      // plain barrier is cheaper than one that carries a verdict), before
-      // the failed stage's slot could be issued again.
-      mbar_wait_or_flag(bars_s + 8u * (s % C::NB), (s / C::NB) & 1, kWaitLimitNs, failed);
-      __syncthreads();
-      if (i % 3 == 0 && __builtin_expect(*failed, 0)) goto wait_failed;
+      // overwrite (ring_wait; a stage that did not land is seen before its
+      // barrier is armed again, SU - PF = 5 stages later).
+      if (ring_wait(bars_s + 8u * (s % C::NB), (s / C::NB) & 1, kWaitLimitNs, failed,
+                    i % kRingLook == 0))
+        goto wait_failed;
       if (tid == 0 && s + C::PF < NS) issue(s + C::PF);
       // Front plane (j+4) into the queue.
       const int fslot = (C::SU == 9) ? p : (s % C::SU);
@@ -761,6 +760,7 @@ __device__ __forceinline__ void sweep_cta(const CUtensorMap *tm_u,
       }
     }
   }
+  if (ring_failed(failed)) goto wait_failed;  // one of the last stages
   if constexpr (C::kScaled) {
     // Largest |u_next| of the step, for the scale of the step after it.
 #pragma unroll
@@ -778,10 +778,7 @@ wait_failed:
     // TMA write lands in shared memory after this CTA has exited.
     if (tid == 0) {
       atomicCAS(&a.desc->error, 0, kErrTimeout);
-      const int issued = min(NS, max(C::SU, s + C::PF));
-      for (int t = max(0, s - kR); t < issued; ++t)
-        if (!mbar_wait_bounded(&bars[t % C::NB], (t / C::NB) & 1, kWaitLimitNs))
-          break;
+      ring_drain<C::NB>(bars, max(0, s - kR), min(NS, max(C::SU, s + C::PF)), kWaitLimitNs);
     }
     __syncthreads();
   }
@@ -1076,7 +1073,7 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
     q[p] = make_float4(fa.x, fa.y, fb.x, fb.y);
     if (p == kR - 1) {
       __syncthreads();
-      if (*failed) goto wait_failed;
+      if (ring_failed(failed)) goto wait_failed;
       if (tid == 0)
         for (int t = C::SU; t < 2 * kR + C::PF && t < NS; ++t) issue(t, t - C::SU);
     }
@@ -1088,11 +1085,11 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
       s = s0 + i;
       if (s >= NS) break;
       // One barrier per plane: stage s has landed for every thread, and every
-      // thread is done with plane s-1, whose slots the next issue reuses. A
-      // wait that gave up is looked for every third plane (see sweep_cta).
-      mbar_wait_or_flag(bars_s + 8u * p, i == 0 ? par9 : par9 ^ 1u, kWaitLimitNs, failed);
-      __syncthreads();
-      if (i % 3 == 0 && __builtin_expect(*failed, 0)) goto wait_failed;
+      // thread is done with plane s-1, whose slots the next issue reuses (see
+      // sweep_cta).
+      if (ring_wait(bars_s + 8u * p, i == 0 ? par9 : par9 ^ 1u, kWaitLimitNs, failed,
+                    i % kRingLook == 0))
+        goto wait_failed;
       if (tid == 0 && s < ns_issue) issue(s + C::PF, (p + C::PF) % 9);
       // The last plane's receivers: no barrier of their own, which in this
       // loop, even where no receiver is, cost 100 cycles of 710 a plane.
@@ -1177,6 +1174,7 @@ __device__ __forceinline__ void sweep_cta_tc(const CUtensorMap *tm_u,
       }
     }
   }
+  if (ring_failed(failed)) goto wait_failed;  // one of the last stages
   if (rz == ze - 1) {  // receivers on the last plane
     __syncthreads();
     record(rz);
@@ -1197,10 +1195,7 @@ wait_failed:
     // TMA write lands in shared memory after this CTA has exited.
     if (tid == 0) {
       atomicCAS(&a.desc->error, 0, kErrTimeout);
-      const int issued = min(NS, max(C::SU, s + C::PF));
-      for (int t = max(0, s - kR); t < issued; ++t)
-        if (!mbar_wait_bounded(&bars[t % C::NB], (t / C::NB) & 1, kWaitLimitNs))
-          break;
+      ring_drain<C::NB>(bars, max(0, s - kR), min(NS, max(C::SU, s + C::PF)), kWaitLimitNs);
     }
     __syncthreads();
   }

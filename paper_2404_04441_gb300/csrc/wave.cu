@@ -142,13 +142,43 @@ Variant pick_variant(int storage, int which) {
 
 __global__ void advance_kernel(StepDesc *d, int k) { d->n += k; }
 
-// Waits on a barrier no one arrives on; records 2 if the wait gave up.
-__global__ void selftest_wait_kernel(uint64_t limit_ns, int *out) {
-  __shared__ uint64_t bar;
-  mbar_init(&bar, 1);
-  fence_barrier_init();
-  const bool done = mbar_wait_bounded(&bar, 0, limit_ns);
-  *out = done ? 1 : 2;
+// The bounded waits on stages that never come. Block 0: mbar_wait_bounded on a
+// barrier no one arrives on. Every other block: the ring of a sweep, its loop
+// and its checks, over `len` stages of which stage `lost` never arrives, for
+// each lost < len <= kSelftestLen. Records 2 where the loss was seen, else 1.
+constexpr int kSelftestLen = 10;
+constexpr int kSelftestBlocks = 1 + kSelftestLen * (kSelftestLen + 1) / 2;
+
+__global__ void __launch_bounds__(128) selftest_wait_kernel(uint64_t limit_ns, int *out) {
+  constexpr int NB = 9, PF = 4;
+  __shared__ uint64_t bars[NB];
+  __shared__ int flag;
+  volatile int *failed = &flag;
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < NB; ++b) mbar_init(&bars[b], 1);
+    fence_barrier_init();
+    *failed = 0;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    const bool done = mbar_wait_bounded(&bars[0], 0, limit_ns);
+    if (threadIdx.x == 0) out[0] = done ? 1 : 2;
+    return;
+  }
+  int len = 1, lost = blockIdx.x - 1;
+  while (lost >= len) lost -= len++;
+  auto issue = [&](int t) {
+    if (threadIdx.x == 0 && t < len && t != lost) mbar_arrive_expect_tx(&bars[t % NB], 0);
+  };
+  for (int t = 0; t < PF; ++t) issue(t);
+  bool seen = false;
+  for (int s = 0; s < len && !seen; ++s) {
+    seen = ring_wait(smem_addr(&bars[s % NB]), (s / NB) & 1, limit_ns, failed,
+                     s % kRingLook == 0);
+    if (!seen) issue(s + PF);
+  }
+  if (!seen) seen = ring_failed(failed);
+  if (threadIdx.x == 0) out[blockIdx.x] = seen ? 2 : 1;
 }
 
 }  // namespace
@@ -1319,20 +1349,21 @@ int wave_get_launch_info(const wave_ctx *c, int *tile_x, int *tile_y,
 int wave_selftest_wait(int64_t limit_ns, void *stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   limit_ns = std::min<int64_t>(std::max<int64_t>(limit_ns, 1000000), 10000000000ll);
-  int *d = nullptr;
-  WAVE_TRY_CUDA(cudaMalloc(&d, sizeof(int)));
-  int h = 0;
-  cudaError_t e = cudaMemsetAsync(d, 0, sizeof(int), st);
+  int *d = nullptr, h[kSelftestBlocks] = {};
+  WAVE_TRY_CUDA(cudaMalloc(&d, sizeof(h)));
+  cudaError_t e = cudaMemsetAsync(d, 0, sizeof(h), st);
   if (e == cudaSuccess) {
-    selftest_wait_kernel<<<1, 1, 0, st>>>((uint64_t)limit_ns, d);
+    selftest_wait_kernel<<<kSelftestBlocks, 128, 0, st>>>((uint64_t)limit_ns, d);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&h, d, sizeof(int), cudaMemcpyDeviceToHost, st);
+    e = cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(d);
   if (e != cudaSuccess) return cuda_status(e);
-  return h == 2 ? WAVE_ETIMEOUT : WAVE_ECUDA;
+  for (int v : h)
+    if (v != 2) return WAVE_ECUDA;
+  return WAVE_ETIMEOUT;
 }
 
 }  // extern "C"
