@@ -1141,6 +1141,13 @@ inline int cpml_batch_group(const CpmlPlan &p) {
 }
 // Blocks of a shot in launch `which` (0..5) of its group.
 int cpml_batch_blocks(const CpmlBatchShot &s, int which);
+// Launches of a group's step, one after another: its line passes and the shell
+// receivers.
+inline int cpml_batch_launches(const int blocks[6]) {
+  int n = 1;
+  for (int i = 0; i < 6; ++i) n += blocks[i] > 0;
+  return n;
+}
 // One batch step's launches over a group's n shots (layer.cu); blocks: their
 // totals per launch; rec_blocks: blocks per shot for its receivers.
 void cpml_batch_step(int storage, int group, const CpmlBatchShot *shots, int n,

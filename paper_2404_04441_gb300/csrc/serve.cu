@@ -61,12 +61,22 @@ struct Group {
 };
 
 // Layered shots of one storage type and one form of the layer's passes:
-// neighbours in the batch table, one launch each.
+// neighbours in the batch table, launched together.
 struct LayerGroup {
   int kind, form, first, count;
   int blocks[6];
   int rec_blocks;  // per shot, for its shell receivers
+  int lane;        // of kLanes
 };
+
+// The groups of a step touch different shots, so they run side by side: lane 0
+// is the server's stream, lane i a stream of priority -i, joined to it around
+// each step; the longest chain of launches goes to the highest. Six FP32 shots
+// of 200 steps, one group after another and now: 64 to 84 cells a side, layers
+// of 6 to 20 cells 33.1 -> 19.9 ms; 200 to 220 a side, layers of 8, 12 and 16
+// 84.1 -> 74.8 (79.9 without the priorities). Line walks of every width in one
+// launch per axis took 23.2 and 78.8.
+constexpr int kLanes = 4;
 
 template <class C>
 Kind make_kind() {
@@ -192,6 +202,9 @@ struct serve_ctx {
   CpmlBatchShot *d_layer[kKinds] = {nullptr, nullptr, nullptr};
   std::vector<CpmlBatchShot> h_layer[kKinds];
   std::vector<LayerGroup> layer_groups;
+  int lanes = 0;  // the groups' lanes, 1 or more streams
+  cudaStream_t lane[kLanes] = {};
+  cudaEvent_t fork = nullptr, join[kLanes] = {};
   std::vector<Group> groups;
   bool dirty = true;
   void *d_scan = nullptr;     // 16 bytes: velocity max, invalid count
@@ -489,7 +502,7 @@ int upload_tables(serve_ctx *s) {
     auto &lt = s->h_layer[kd];
     lt.clear();
     for (int form = 0; form < kCpmlGroups; ++form) {
-      LayerGroup lg{kd, form, (int)lt.size(), 0, {}, 1};
+      LayerGroup lg{kd, form, (int)lt.size(), 0, {}, 1, 0};
       for (Request *q : shots) {
         if (q->r.npml <= 0 || cpml_batch_group(q->layer.plan) != form) continue;
         CpmlBatchShot L = q->layer;
@@ -508,8 +521,55 @@ int upload_tables(serve_ctx *s) {
       WAVE_TRY_CUDA(cudaMemcpyAsync(s->d_layer[kd], lt.data(), lt.size() * sizeof(CpmlBatchShot),
                                     cudaMemcpyHostToDevice, s->stream));
   }
+  // longest chains of launches first, each to the lane with the fewest so far,
+  // from the lane of the highest priority down
+  std::stable_sort(s->layer_groups.begin(), s->layer_groups.end(),
+                   [](const LayerGroup &a, const LayerGroup &b) {
+                     return cpml_batch_launches(a.blocks) > cpml_batch_launches(b.blocks);
+                   });
+  int load[kLanes] = {};
+  s->lanes = std::min(kLanes, (int)s->layer_groups.size());
+  for (LayerGroup &g : s->layer_groups) {
+    g.lane = s->lanes - 1;
+    for (int i = g.lane; i >= 0; --i)
+      if (load[i] < load[g.lane]) g.lane = i;
+    load[g.lane] += cpml_batch_launches(g.blocks);
+  }
   s->dirty = false;
   return WAVE_OK;
+}
+
+// The layer's terms and shell receivers of batch step k, after its sweeps.
+int launch_layers(serve_ctx *s, long long k) {
+  if (s->lanes > 1) WAVE_TRY_CUDA(cudaEventRecord(s->fork, s->stream));
+  for (int i = 1; i < s->lanes; ++i)
+    WAVE_TRY_CUDA(cudaStreamWaitEvent(s->lane[i], s->fork, 0));
+  for (const LayerGroup &g : s->layer_groups)
+    cpml_batch_step(g.kind, g.form, s->d_layer[g.kind] + g.first, g.count, g.blocks,
+                    g.rec_blocks, k, s->lane[g.lane]);
+  for (int i = 1; i < s->lanes; ++i) {
+    WAVE_TRY_CUDA(cudaEventRecord(s->join[i], s->lane[i]));
+    WAVE_TRY_CUDA(cudaStreamWaitEvent(s->stream, s->join[i], 0));
+  }
+  return WAVE_OK;
+}
+
+int create_lanes(serve_ctx *s) {
+  s->lane[0] = s->stream;
+  WAVE_TRY_CUDA(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
+  for (int i = 1; i < kLanes; ++i) {
+    WAVE_TRY_CUDA(cudaStreamCreateWithPriority(&s->lane[i], cudaStreamNonBlocking, -i));
+    WAVE_TRY_CUDA(cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming));
+  }
+  return WAVE_OK;
+}
+
+void destroy_lanes(serve_ctx *s) {
+  for (int i = 1; i < kLanes; ++i) {
+    if (s->lane[i]) cudaStreamDestroy(s->lane[i]);
+    if (s->join[i]) cudaEventDestroy(s->join[i]);
+  }
+  if (s->fork) cudaEventDestroy(s->fork);
 }
 
 // Complete a resident shot whose steps are all done (stream synchronized).
@@ -600,13 +660,13 @@ void engine_main(serve_ctx *s) {
       for (const Group &g : s->groups)
         kind_of(g.kind).launch(g.ctas, s->stream, s->d_table[g.kind] + g.first,
                                g.count, s->k + kk, g.co);
-      for (const LayerGroup &lg : s->layer_groups)
-        cpml_batch_step(lg.kind, lg.form, s->d_layer[lg.kind] + lg.first, lg.count, lg.blocks,
-                        lg.rec_blocks, s->k + kk, s->stream);
+      status = launch_layers(s, s->k + kk);
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (status == WAVE_OK && e != cudaSuccess) status = cuda_status(e);
+    // a step cut short may have left a lane that the stream does not wait for
+    for (int i = 1; i < s->lanes && status != WAVE_OK; ++i) cudaStreamSynchronize(s->lane[i]);
     s->k += K;
     {
       std::lock_guard<std::mutex> lk(s->mu);
@@ -720,6 +780,7 @@ int serve_create(size_t hbm_budget_bytes, int max_slots, void *stream,
                                  sizeof(CpmlBatchShot) * (size_t)max_slots));
   }
   if (e == WAVE_OK) e = cuda_status(device_malloc(&s->d_scan, 16));
+  if (e == WAVE_OK) e = create_lanes(s.get());
   if (e == WAVE_OK) {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
@@ -739,6 +800,7 @@ int serve_create(size_t hbm_budget_bytes, int max_slots, void *stream,
       cudaFree(s->d_layer[kd]);
     }
     cudaFree(s->d_scan);
+    destroy_lanes(s.get());
     if (s->pool) cudaMemPoolDestroy(s->pool);
     if (s->own_stream) cudaStreamDestroy(s->stream);
     return e;
@@ -820,6 +882,7 @@ void serve_destroy(serve_ctx *s) {
     cudaFree(s->d_layer[kd]);
   }
   cudaFree(s->d_scan);
+  destroy_lanes(s);
   if (s->pool) cudaMemPoolDestroy(s->pool);
   if (s->own_stream) cudaStreamDestroy(s->stream);
   delete s;
