@@ -224,7 +224,7 @@ int serve_alloc(serve_ctx *s, void **p, size_t bytes) {
   if (s->fault_alloc >= 0 && s->allocs++ == s->fault_alloc) return WAVE_ENOMEM;
   bytes = std::max<size_t>(bytes, 256);
   cudaError_t e = cudaMallocFromPoolAsync(p, bytes, s->pool, s->stream);
-  if (e == cudaErrorMemoryAllocation && drop_kept_workspace(s->device)) {
+  if (e == cudaErrorMemoryAllocation && drop_kept_workspace()) {
     cudaGetLastError();
     e = cudaMallocFromPoolAsync(p, bytes, s->pool, s->stream);
   }

@@ -196,7 +196,8 @@ struct wave_ctx {
   cudaStream_t stream = nullptr;
   cudaStream_t capture_stream = nullptr;
   int device = 0;
-  bool counted = false;  // among its device's contexts (KeptWork)
+  bool counted = false;  // among those of its CUDA context (KeptWork)
+  unsigned long long home = 0;  // that context
   void *base = nullptr;  // one allocation: both wavefields, c, desc, scratch
   void *buf[2] = {nullptr, nullptr};  // buf[cur] = u, buf[cur ^ 1] = u_prev
   float *c = nullptr;
@@ -243,57 +244,91 @@ struct wave_ctx {
   int *d_nsrec = nullptr;  // their count (device: graphs stay valid)
 };
 
-// The gradient's workspace, kept between calls: one block per device, of at
-// most 1/16 of its memory, while a context lives there. Mapping and unmapping
-// it on each call cost 4.1 ms of a gradient at 256^3 x 160 steps (6.3 GB in 14
-// allocations; 36.4 -> 31.1 ms) and a call of one step 3.8 ms. A call takes
-// the block out, so calls that run at once (other threads, other streams) have
-// blocks of their own, and gives it back after its last stream synchronisation;
-// what does not fit, or a second block, is freed. An allocation of the library
-// that fails frees the kept block and tries again; so does the end of the last
-// context.
+// The gradient's workspace, kept between calls: one block per CUDA context, of
+// at most 1/16 of its device's memory, while a wave_ctx lives there. Mapping and
+// unmapping it on each call cost 4.1 ms of a gradient at 256^3 x 160 steps (6.3
+// GB in 14 allocations; 36.4 -> 31.1 ms) and a call of one step 3.8 ms. A call
+// takes the block out, so calls that run at once (other threads, other streams)
+// have blocks of their own, and gives it back after its last stream
+// synchronisation; what does not fit, or a second block, is freed. An allocation
+// of the library that fails frees the kept block and tries again; so does the
+// end of the last wave_ctx. The blocks are found by the CUDA context's id, which
+// no later context has: one that cudaDeviceReset took is never handed out.
 namespace {
 
-constexpr int kWorkDevices = 64;
-
 struct KeptWork {
-  std::mutex mu;
-  void *p[kWorkDevices] = {};
-  size_t cap[kWorkDevices] = {};
-  int contexts[kWorkDevices] = {};
+  unsigned long long home = 0;  // the CUDA context
+  int contexts = 0;             // wave_ctx alive there
+  void *p = nullptr;
+  size_t cap = 0;
 };
-KeptWork g_work;
+constexpr int kWorkContexts = 64;
+std::mutex g_work_mu;
+KeptWork g_work[kWorkContexts];
 
-// Frees a device's kept block (mu held).
-bool drop_locked(int dev) {
-  if (!g_work.p[dev]) return false;
-  cudaFree(g_work.p[dev]);
-  g_work.p[dev] = nullptr;
-  g_work.cap[dev] = 0;
+// Id of the current CUDA context (after a runtime call on its device).
+unsigned long long cuda_context_id() {
+  static const auto get = [] {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    return cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) ==
+                       cudaSuccess &&
+                   q == cudaDriverEntryPointSuccess
+               ? reinterpret_cast<PFN_cuCtxGetId_v12000>(p)
+               : nullptr;
+  }();
+  unsigned long long id = 0;
+  return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// The entry of a CUDA context, nullptr if no wave_ctx lives there (g_work_mu
+// held).
+KeptWork *work_of(unsigned long long home) {
+  for (KeptWork &w : g_work)
+    if (w.contexts > 0 && w.home == home) return &w;
+  return nullptr;
+}
+
+// Frees a kept block (g_work_mu held).
+bool drop_locked(KeptWork &w) {
+  if (!w.p) return false;
+  cudaFree(w.p);
+  w.p = nullptr;
+  w.cap = 0;
   return true;
 }
 
-void count_context(int dev, int by) {
-  if (dev < 0 || dev >= kWorkDevices) return;
-  std::lock_guard<std::mutex> lock(g_work.mu);
-  if ((g_work.contexts[dev] += by) == 0) drop_locked(dev);
+// Counts a wave_ctx in; false (nothing is kept for it) with no entry left.
+bool enter_context(unsigned long long home) {
+  std::lock_guard<std::mutex> lock(g_work_mu);
+  KeptWork *w = work_of(home);
+  for (int i = 0; i < kWorkContexts && !w; ++i)
+    if (g_work[i].contexts == 0) w = &g_work[i];
+  if (!w) return false;
+  w->home = home;
+  w->contexts++;
+  return true;
+}
+
+void leave_context(unsigned long long home) {
+  std::lock_guard<std::mutex> lock(g_work_mu);
+  KeptWork *w = work_of(home);
+  if (w && --w->contexts == 0) drop_locked(*w);
 }
 
 }  // namespace
 
 namespace gbw {
 
-bool drop_kept_workspace(int dev) {
-  if (dev < 0 || dev >= kWorkDevices) return false;
-  std::lock_guard<std::mutex> lock(g_work.mu);
-  return drop_locked(dev);
+bool drop_kept_workspace() {
+  std::lock_guard<std::mutex> lock(g_work_mu);
+  KeptWork *w = work_of(cuda_context_id());
+  return w && drop_locked(*w);
 }
 
 cudaError_t device_malloc(void **p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes);
-  int dev = -1;
-  if (e == cudaErrorMemoryAllocation && cudaGetDevice(&dev) == cudaSuccess &&
-      drop_kept_workspace(dev)) {
+  if (e == cudaErrorMemoryAllocation && drop_kept_workspace()) {
     cudaGetLastError();
     e = cudaMalloc(p, bytes);
   }
@@ -308,7 +343,7 @@ size_t round_up256(size_t x) { return (x + 255) & ~size_t(255); }
 
 int ensure_for(const wave_ctx *c, DeviceBuf &b, size_t bytes) {
   const int st = ensure(b, bytes, c->stream);
-  if (st != WAVE_ENOMEM || !drop_kept_workspace(c->device)) return st;
+  if (st != WAVE_ENOMEM || !drop_kept_workspace()) return st;
   cudaGetLastError();
   return ensure(b, bytes, c->stream);
 }
@@ -575,7 +610,7 @@ void wave_destroy(wave_ctx *c) {
   free_cpml(c);
   cudaFree(c->srec.p);
   cudaFree(c->d_nsrec);
-  if (c->counted) count_context(c->device, -1);
+  if (c->counted) leave_context(c->home);
   delete c;
 }
 
@@ -619,13 +654,13 @@ static int alloc_context(wave_ctx *c) {
   const char *ev = std::getenv("GBWAVE_VARIANT");
   c->var = pick_variant(c->storage, ev ? std::atoi(ev) : 0);
   WAVE_TRY_CUDA(cudaGetDevice(&c->device));
-  count_context(c->device, 1);
-  c->counted = true;
   WAVE_TRY_CUDA(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount,
                                        c->device));
   WAVE_TRY_CUDA(cudaStreamCreateWithFlags(&c->capture_stream,
                                           cudaStreamNonBlocking));
   WAVE_TRY_CUDA(cudaEventCreateWithFlags(&c->ev_aux, cudaEventDisableTiming));
+  c->home = cuda_context_id();  // current since the stream's creation
+  c->counted = enter_context(c->home);
   const size_t fbytes = field_bytes(c);
   const size_t off1 = round_up256(fbytes), offc = off1 + round_up256(fbytes);
   const size_t offd = offc + round_up256(bytes);
@@ -1501,22 +1536,22 @@ __global__ void grad_assemble_kernel(const double *gacc, const float *c,
 // A gradient call's device buffers: asked for one by one, then placed in one
 // block (KeptWork). Freed on scope exit, or kept after done().
 struct Workspace {
-  int dev;
+  unsigned long long home;
   void *block = nullptr;
   size_t cap = 0, bytes = 0;
   bool keep = false;
   std::vector<std::pair<void **, size_t>> asked;
 
-  explicit Workspace(int d) : dev(d) {}
+  explicit Workspace(const wave_ctx *c) : home(c->home) {}
   ~Workspace() {
     if (!block) return;
     if (keep) {
       size_t all = 0, avail = 0;
-      std::lock_guard<std::mutex> lock(g_work.mu);
-      if (dev >= 0 && dev < kWorkDevices && !g_work.p[dev] && g_work.contexts[dev] > 0 &&
-          cudaMemGetInfo(&avail, &all) == cudaSuccess && cap <= all / 16) {
-        g_work.p[dev] = block;
-        g_work.cap[dev] = cap;
+      std::lock_guard<std::mutex> lock(g_work_mu);
+      KeptWork *w = work_of(home);
+      if (w && !w->p && cudaMemGetInfo(&avail, &all) == cudaSuccess && cap <= all / 16) {
+        w->p = block;
+        w->cap = cap;
         return;
       }
     }
@@ -1528,15 +1563,14 @@ struct Workspace {
     bytes += (std::max<size_t>(n, 1) + 511) & ~size_t(511);
   }
   int place() {
-    if (dev >= 0 && dev < kWorkDevices) {
-      std::lock_guard<std::mutex> lock(g_work.mu);
-      if (g_work.cap[dev] >= bytes) {
-        block = g_work.p[dev];
-        cap = g_work.cap[dev];
-        g_work.p[dev] = nullptr;
-        g_work.cap[dev] = 0;
-      } else {
-        drop_locked(dev);  // too small: this call's block is kept instead
+    {
+      std::lock_guard<std::mutex> lock(g_work_mu);
+      KeptWork *w = work_of(home);
+      if (w && w->cap >= bytes) {
+        block = std::exchange(w->p, nullptr);
+        cap = std::exchange(w->cap, 0);
+      } else if (w) {
+        drop_locked(*w);  // too small: this call's block is kept instead
       }
     }
     if (!block) {
@@ -1569,7 +1603,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   const size_t fb = fe * 4;
   const int ncp = (N + K - 1) / K;
   const size_t tn = (size_t)N * nrec;
-  Workspace mem(c->device);
+  Workspace mem(c);
   float *ckpt, *dbuf, *padj[2], *trd, *res, *inj, *wl, *ghi, *glo;
   double *gacc, *dmis;
   StepDesc *dadj, *dfwd;

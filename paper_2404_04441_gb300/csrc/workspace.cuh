@@ -8,7 +8,7 @@ namespace gbw {
 // cudaMalloc on the current device; if that runs out of memory, frees the kept
 // workspace and tries again.
 cudaError_t device_malloc(void **p, size_t bytes);
-// Frees a device's kept workspace; false if there is none.
-bool drop_kept_workspace(int device);
+// Frees the current CUDA context's kept workspace; false if there is none.
+bool drop_kept_workspace();
 
 }  // namespace gbw
