@@ -309,10 +309,11 @@ int wave_selftest_wait(int64_t limit_ns, void *stream);
  *   ckpt_every   steps per checkpoint segment (>= 1); device memory holds
  *                2 * ceil(nsteps/ckpt_every) + 2 * ckpt_every + 6 float32
  *                fields (ckpt_every + 8 when one segment covers nsteps; the
- *                FP64 time sum counts as two), plus the traces; up to 1/16 of
- *                the device's memory of it is kept for the next call, until
- *                the device's last context is destroyed or another allocation
- *                of the library needs it
+ *                FP64 time sum counts as two), plus the traces. Up to 1/16 of
+ *                the device's memory of it is kept for the next call until the
+ *                device's last context is destroyed; of that, all but 1/256 of
+ *                the device's memory goes to any allocation of the process
+ *                that would not fit otherwise, and the rest to the library's
  *   grad_v2      nx*ny*nz float32 output (host or device), dense, x fastest
  *   traces       optional nsteps*nrec float32 output of the forward traces
  * FP32 storage and the default kernel variant only (else WAVE_ENOTSUP). The

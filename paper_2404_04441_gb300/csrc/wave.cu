@@ -244,16 +244,22 @@ struct wave_ctx {
   int *d_nsrec = nullptr;  // their count (device: graphs stay valid)
 };
 
-// The gradient's workspace, kept between calls: one block per CUDA context, of
-// at most 1/16 of its device's memory, while a wave_ctx lives there. Mapping and
-// unmapping it on each call cost 4.1 ms of a gradient at 256^3 x 160 steps (6.3
-// GB in 14 allocations; 36.4 -> 31.1 ms) and a call of one step 3.8 ms. A call
-// takes the block out, so calls that run at once (other threads, other streams)
-// have blocks of their own, and gives it back after its last stream
-// synchronisation; what does not fit, or a second block, is freed. An allocation
-// of the library that fails frees the kept block and tries again; so does the
-// end of the last wave_ctx. The blocks are found by the CUDA context's id, which
-// no later context has: one that cudaDeviceReset took is never handed out.
+// The gradient's workspace, kept between calls while a wave_ctx lives in the CUDA
+// context: mapping and unmapping it on each call cost 4.1 ms of a gradient at
+// 256^3 x 160 steps (6.3 GB in 14 allocations; 36.4 -> 31.1 ms) and a call of one
+// step 3.8 ms.
+//  * Up to 1/256 of the device's memory: one block. A call takes it out, so
+//    calls that run at once (other threads, other streams) have blocks of their
+//    own, and gives it back after its last stream synchronisation; a second block
+//    is freed. An allocation of the library that fails frees the kept block and
+//    tries again; so does the end of the last wave_ctx.
+//  * From there to 1/16: memory of a pool that keeps that much, which the driver
+//    takes back when any allocation of the process runs out. A pool grows and
+//    shrinks slowly (0.86 and 1.5 ms per GB, cudaMalloc and cudaFree 0.04 and
+//    0.37), so it serves from the second such call on.
+//  * Larger ones are allocated and freed by each call.
+// The entries are found by the CUDA context's id, which no later context has:
+// memory that cudaDeviceReset took is never handed out.
 namespace {
 
 struct KeptWork {
@@ -261,6 +267,9 @@ struct KeptWork {
   int contexts = 0;             // wave_ctx alive there
   void *p = nullptr;
   size_t cap = 0;
+  size_t memory = 0;  // of the device
+  bool pooled = false;  // a call has been of a size for the pool
+  cudaMemPool_t pool = nullptr;
 };
 constexpr int kWorkContexts = 64;
 std::mutex g_work_mu;
@@ -304,7 +313,8 @@ bool enter_context(unsigned long long home) {
   KeptWork *w = work_of(home);
   for (int i = 0; i < kWorkContexts && !w; ++i)
     if (g_work[i].contexts == 0) w = &g_work[i];
-  if (!w) return false;
+  size_t avail = 0;
+  if (!w || (w->memory == 0 && cudaMemGetInfo(&avail, &w->memory) != cudaSuccess)) return false;
   w->home = home;
   w->contexts++;
   return true;
@@ -313,7 +323,27 @@ bool enter_context(unsigned long long home) {
 void leave_context(unsigned long long home) {
   std::lock_guard<std::mutex> lock(g_work_mu);
   KeptWork *w = work_of(home);
-  if (w && --w->contexts == 0) drop_locked(*w);
+  if (!w || --w->contexts > 0) return;
+  drop_locked(*w);
+  if (w->pool) cudaMemPoolDestroy(w->pool);
+  *w = KeptWork{};
+}
+
+// The entry's pool (g_work_mu held), nullptr if there can be none.
+cudaMemPool_t pool_locked(KeptWork &w, int device) {
+  if (w.pool) return w.pool;
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  cudaMemPool_t pool = nullptr;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  cuuint64_t keep = w.memory / 16;
+  cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  return w.pool = pool;
 }
 
 }  // namespace
@@ -1536,20 +1566,24 @@ __global__ void grad_assemble_kernel(const double *gacc, const float *c,
 // A gradient call's device buffers: asked for one by one, then placed in one
 // block (KeptWork). Freed on scope exit, or kept after done().
 struct Workspace {
-  unsigned long long home;
+  const wave_ctx *c;
   void *block = nullptr;
   size_t cap = 0, bytes = 0;
-  bool keep = false;
+  bool keep = false, pooled = false;
   std::vector<std::pair<void **, size_t>> asked;
 
-  explicit Workspace(const wave_ctx *c) : home(c->home) {}
+  explicit Workspace(const wave_ctx *ctx) : c(ctx) {}
   ~Workspace() {
     if (!block) return;
+    if (pooled) {
+      if (!keep) cudaDeviceSynchronize();  // both streams may still use it
+      cudaFreeAsync(block, c->stream);
+      return;
+    }
     if (keep) {
-      size_t all = 0, avail = 0;
       std::lock_guard<std::mutex> lock(g_work_mu);
-      KeptWork *w = work_of(home);
-      if (w && !w->p && cudaMemGetInfo(&avail, &all) == cudaSuccess && cap <= all / 16) {
+      KeptWork *w = c->counted ? work_of(c->home) : nullptr;
+      if (w && !w->p && cap <= w->memory / 256) {
         w->p = block;
         w->cap = cap;
         return;
@@ -1563,14 +1597,28 @@ struct Workspace {
     bytes += (std::max<size_t>(n, 1) + 511) & ~size_t(511);
   }
   int place() {
-    {
+    cudaMemPool_t pool = nullptr;
+    if (c->counted) {
       std::lock_guard<std::mutex> lock(g_work_mu);
-      KeptWork *w = work_of(home);
-      if (w && w->cap >= bytes) {
-        block = std::exchange(w->p, nullptr);
-        cap = std::exchange(w->cap, 0);
-      } else if (w) {
-        drop_locked(*w);  // too small: this call's block is kept instead
+      KeptWork &w = *work_of(c->home);
+      if (bytes <= w.memory / 256) {
+        if (w.cap >= bytes) {
+          block = std::exchange(w.p, nullptr);
+          cap = std::exchange(w.cap, 0);
+        } else {
+          drop_locked(w);  // too small: this call's block is kept instead
+        }
+      } else if (bytes <= w.memory / 16) {
+        if (w.pooled) pool = pool_locked(w, c->device);
+        w.pooled = true;
+      }
+    }
+    if (pool) {
+      if (cudaMallocFromPoolAsync(&block, bytes, pool, c->stream) == cudaSuccess) {
+        pooled = true;
+      } else {
+        cudaGetLastError();
+        block = nullptr;
       }
     }
     if (!block) {
