@@ -463,6 +463,27 @@ int admit(serve_ctx *s, Request *q) {
   return WAVE_OK;
 }
 
+// The lanes beside the server's stream, created for the first batch of several
+// groups (0.7 ms).
+int create_lanes(serve_ctx *s) {
+  if (!s->fork) WAVE_TRY_CUDA(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
+  for (int i = 1; i < kLanes; ++i) {
+    if (!s->lane[i])
+      WAVE_TRY_CUDA(cudaStreamCreateWithPriority(&s->lane[i], cudaStreamNonBlocking, -i));
+    if (!s->join[i])
+      WAVE_TRY_CUDA(cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming));
+  }
+  return WAVE_OK;
+}
+
+void destroy_lanes(serve_ctx *s) {
+  for (int i = 1; i < kLanes; ++i) {
+    if (s->lane[i]) cudaStreamDestroy(s->lane[i]);
+    if (s->join[i]) cudaEventDestroy(s->join[i]);
+  }
+  if (s->fork) cudaEventDestroy(s->fork);
+}
+
 // Order the resident shots by (storage, spacing), cut them into launch
 // groups and upload the batch tables.
 int upload_tables(serve_ctx *s) {
@@ -529,6 +550,10 @@ int upload_tables(serve_ctx *s) {
                    });
   int load[kLanes] = {};
   s->lanes = std::min(kLanes, (int)s->layer_groups.size());
+  if (s->lanes > 1 && create_lanes(s) != WAVE_OK) {
+    cudaGetLastError();
+    s->lanes = 1;
+  }
   for (LayerGroup &g : s->layer_groups) {
     g.lane = s->lanes - 1;
     for (int i = g.lane; i >= 0; --i)
@@ -552,24 +577,6 @@ int launch_layers(serve_ctx *s, long long k) {
     WAVE_TRY_CUDA(cudaStreamWaitEvent(s->stream, s->join[i], 0));
   }
   return WAVE_OK;
-}
-
-int create_lanes(serve_ctx *s) {
-  s->lane[0] = s->stream;
-  WAVE_TRY_CUDA(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
-  for (int i = 1; i < kLanes; ++i) {
-    WAVE_TRY_CUDA(cudaStreamCreateWithPriority(&s->lane[i], cudaStreamNonBlocking, -i));
-    WAVE_TRY_CUDA(cudaEventCreateWithFlags(&s->join[i], cudaEventDisableTiming));
-  }
-  return WAVE_OK;
-}
-
-void destroy_lanes(serve_ctx *s) {
-  for (int i = 1; i < kLanes; ++i) {
-    if (s->lane[i]) cudaStreamDestroy(s->lane[i]);
-    if (s->join[i]) cudaEventDestroy(s->join[i]);
-  }
-  if (s->fork) cudaEventDestroy(s->fork);
 }
 
 // Complete a resident shot whose steps are all done (stream synchronized).
@@ -767,6 +774,7 @@ int serve_create(size_t hbm_budget_bytes, int max_slots, void *stream,
     WAVE_TRY_CUDA(cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking));
     s->own_stream = true;
   }
+  s->lane[0] = s->stream;
   int e = WAVE_OK;
   for (int kd = 0; kd < kKinds && e == WAVE_OK; ++kd) {
     const Kind &k = kind_of(kd);
@@ -780,7 +788,6 @@ int serve_create(size_t hbm_budget_bytes, int max_slots, void *stream,
                                  sizeof(CpmlBatchShot) * (size_t)max_slots));
   }
   if (e == WAVE_OK) e = cuda_status(device_malloc(&s->d_scan, 16));
-  if (e == WAVE_OK) e = create_lanes(s.get());
   if (e == WAVE_OK) {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
@@ -800,7 +807,6 @@ int serve_create(size_t hbm_budget_bytes, int max_slots, void *stream,
       cudaFree(s->d_layer[kd]);
     }
     cudaFree(s->d_scan);
-    destroy_lanes(s.get());
     if (s->pool) cudaMemPoolDestroy(s->pool);
     if (s->own_stream) cudaStreamDestroy(s->stream);
     return e;
