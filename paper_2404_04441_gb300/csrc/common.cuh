@@ -377,14 +377,21 @@ bool is_device_ptr(const void *p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Memory that kernels on `device` can read and write in place: its own.
-bool is_memory_of(const void *p, int device) {
+// Whether kernels take a field's rows to or from memory of these attributes: the
+// context device's own, with that device current (a copy may be issued to a
+// stream of another device, a kernel may not).
+inline bool rows_by_kernel(const cudaPointerAttributes &at, int device, int current) {
+  return at.type == cudaMemoryTypeDevice && at.device == device && current == device;
+}
+
+bool rows_by_kernel(const void *p, int device) {
   cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+  int current = -1;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&current) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == device;
+  return rows_by_kernel(at, device, current);
 }
 
 int ensure(DeviceBuf &b, size_t bytes, cudaStream_t st) {

@@ -1161,7 +1161,7 @@ static void launch_to_stored(const wave_ctx *c, void *dst, const float *src, int
 static int copy_field(const wave_ctx *c, float *dst, long long dpitch, const float *src,
                       long long spitch, const float *user) {
   const long long rows = (long long)c->ny * c->nz;
-  if (!is_memory_of(user, c->device)) {
+  if (!rows_by_kernel(user, c->device)) {
     WAVE_TRY_CUDA(cudaMemcpy2DAsync(dst, (size_t)dpitch * 4, src, (size_t)spitch * 4,
                                     (size_t)c->nx * 4, (size_t)rows, cudaMemcpyDefault,
                                     c->stream));
