@@ -1079,6 +1079,24 @@ struct CpmlPlan {
 // 313.
 constexpr long long kCpmlByAxis = 1500000;
 
+inline long long cpml_line_ends(const CpmlGeom &g) {
+  return 2 * ((long long)g.ny * g.nz + (long long)g.nx * g.nz + (long long)g.nx * g.ny);
+}
+
+// Points of line ends (w each) from which the axes take a launch each while
+// another chain of launches runs beside this one (the gradient's recompute and
+// adjoint): clusters of 4 CTAs that fill an SM's registers wait for places
+// together. wave_gradient, checkpoint every 20 steps, us a step in one launch and
+// by axis: 16 cells 144^3 (2.5 M) 113 and 118, 170^3 (3.5 M) 194 and 184; 8 cells
+// 185^3 (2.5 M) 170 and 173, 200^3 (2.9 M) 199 and 193; 10 cells 128 x 128 x 400
+// (3.3 M) 165 and 167, 200^3 (3.4 M) 211 and 205; 16 cells 256^3 (7.9 M),
+// checkpoint every 40, 408 and 365, 512 x 512 x 256 (21 M) 1428 and 1315.
+constexpr long long kCpmlByAxisBeside = 2800000;
+
+inline void cpml_beside(CpmlPlan &p) {
+  p.by_axis |= p.axes == 7 && p.g.w * cpml_line_ends(p.g) >= kCpmlByAxisBeside;
+}
+
 // Takes the plan's form on each axis from the grid and the layer's width
 // (g.npml set), and its tiles.
 inline void cpml_plan_forms(CpmlPlan &p) {
@@ -1091,8 +1109,7 @@ inline void cpml_plan_forms(CpmlPlan &p) {
   for (int ax = 0; ax < 3; ++ax)
     if (cpml_seg_fits(g.npml, n[ax], fstep[ax], sstep[ax])) p.axes |= 1 << ax;
   p.variant = cpml_variant(g.npml);
-  p.by_axis = p.axes == 7 && 2 * ((long long)g.ny * g.nz + (long long)g.nx * g.nz +
-                                  (long long)g.nx * g.ny) >= kCpmlByAxis;
+  p.by_axis = p.axes == 7 && cpml_line_ends(g) >= kCpmlByAxis;
   p.all = cpml_tiles(g.nx, g.ny, g.nz, g.w, -1);
   for (int ax = 0; ax < 3; ++ax) p.one[ax] = cpml_tiles(g.nx, g.ny, g.nz, g.w, ax);
 }

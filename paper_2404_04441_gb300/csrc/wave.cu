@@ -1685,6 +1685,8 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   // with each checkpoint, the recompute steps the saved copies in place, and
   // the adjoint carries its nu, mu slabs.
   const CpmlGeom &cg = c->cp.g;
+  CpmlPlan plan = c->cp;  // of the recompute and the adjoint
+  if (nslot == 2) cpml_beside(plan);
   size_t sl[3] = {0, 0, 0};
   float *ckpt_l = nullptr, *nus[3] = {}, *mus[3] = {};
   if (c->cpml) {
@@ -1700,7 +1702,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
   if ((e = mem.place())) return e;
   // the layer slabs held by a segment's checkpoint (per axis psi, then zeta)
   auto layer_of = [&](int sgm) {
-    CpmlPlan pl = c->cp;
+    CpmlPlan pl = plan;
     CpmlGeom &gg = pl.g;
     float *q = ckpt_l + (sl[0] + sl[1] + sl[2]) * 2 * sgm;
     for (int ax = 0; ax < 3; ++ax) {
@@ -1790,7 +1792,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
       const int me = field_maps(rbuf[b], &rhalo[b], &rtile[b]);
       if (me) return me;
     }
-    const CpmlPlan rp = c->cpml ? layer_of(sgm) : c->cp;
+    const CpmlPlan rp = c->cpml ? layer_of(sgm) : plan;
     int cur = 0;
     for (int n = s0; n < s1; ++n) {
       SweepArgs a = args_d;
@@ -1891,7 +1893,7 @@ int gradient_impl(wave_ctx *c, const wave_shot *shot, int N,
         lp.nus[ax] = nus[ax];
         lp.mus[ax] = mus[ax];
       }
-      cpml_adjoint(c->cp, lp, st);
+      cpml_adjoint(plan, lp, st);
     }
     if (dsrc && k % kGradFold == 0)
       grad_fold_kernel<<<c->sms * 4, 256, 0, st>>>(gacc, ghi, glo, (long long)(fe / 4));

@@ -2,6 +2,9 @@
 walks (GBWAVE_CPML_GENERIC=1), bit for bit: both round each operation alike and
 add the axes' terms in the same order.
 
+In a gradient of several segments the axes take a launch each from 2.8 million
+points of line ends on; a gradient of one segment keeps the single launch there.
+
 Grids: the smallest of two disjoint segments on each axis (2 (npml + 4)); x rows
 that are whole vectors of 4 and not; x too short for the near cells to be rounded
 up to 8, just long enough, and longer; and flat ones of more than 1.5 million
@@ -129,3 +132,13 @@ def test_gradient_by_axis(wave_lib, monkeypatch, npml, nx, ckpt):
     shape = _flat(npml, nx)
     model = _model(shape, npml)
     _same(monkeypatch, lambda: _gradient(wave_lib, shape, npml, 8, ckpt, model))
+
+
+@pytest.mark.parametrize("npml,shape", [(16, (161, 150, 152)), (8, (204, 200, 192))])
+@pytest.mark.parametrize("ckpt", [4, 10])
+def test_gradient_beside_its_recompute(wave_lib, monkeypatch, npml, shape, ckpt):
+    nx, ny, nz = shape
+    ends = 2 * (nx * ny + ny * nz + nx * nz)
+    assert ends * (npml + 4) >= 2800000 and ends < 1500000
+    model = _model(shape, npml)
+    _same(monkeypatch, lambda: _gradient(wave_lib, shape, npml, 10, ckpt, model))
