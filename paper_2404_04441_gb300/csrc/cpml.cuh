@@ -1156,8 +1156,10 @@ constexpr int kCpmlGroups = 2 * kCpmlVariants + 1;
 inline int cpml_batch_group(const CpmlPlan &p) {
   return p.axes == 7 ? p.variant : p.axes ? kCpmlVariants + p.variant : 2 * kCpmlVariants;
 }
-// Blocks of a shot in launch `which` (0..5) of its group.
-int cpml_batch_blocks(const CpmlBatchShot &s, int which);
+// Blocks of a shot in launch `which` (0..5) of its group. by_axis: a launch for
+// each axis although every one is unrolled (as some_axes_group).
+int cpml_batch_blocks(const CpmlBatchShot &s, int which, bool by_axis);
+inline int some_axes_group(int all_axes_group) { return all_axes_group + kCpmlVariants; }
 // Launches of a group's step, one after another: its line passes and the shell
 // receivers.
 inline int cpml_batch_launches(const int blocks[6]) {

@@ -140,10 +140,10 @@ void cpml_adjoint(const CpmlPlan &p, const CpmlPass &a, cudaStream_t st) {
   }
 }
 
-int cpml_batch_blocks(const CpmlBatchShot &s, int which) {
+int cpml_batch_blocks(const CpmlBatchShot &s, int which, bool by_axis) {
   const CpmlPlan &p = s.plan;
   const int ax = which % 3;
-  if (p.axes == 7) return which == 0 ? p.all.start[7] * kCpmlCluster : 0;
+  if (p.axes == 7 && !by_axis) return which == 0 ? p.all.start[7] * kCpmlCluster : 0;
   if ((p.axes >> ax) & 1) return which < 3 ? p.one[ax].start[7] * kCpmlCluster : 0;
   if (which < 3) return 0;
   const int across = ax == 0 ? p.g.ny : p.g.nx, rows = ax == 2 ? p.g.ny : p.g.nz;

@@ -523,13 +523,25 @@ int upload_tables(serve_ctx *s) {
     auto &lt = s->h_layer[kd];
     lt.clear();
     for (int form = 0; form < kCpmlGroups; ++form) {
-      LayerGroup lg{kd, form, (int)lt.size(), 0, {}, 1, 0};
+      std::vector<const Request *> of_form;
+      long long ends = 0;
       for (Request *q : shots) {
         if (q->r.npml <= 0 || cpml_batch_group(q->layer.plan) != form) continue;
+        of_form.push_back(q);
+        ends += cpml_line_ends(q->layer.plan.g);
+      }
+      // Many line ends take a launch per axis, as those of one grid do: the
+      // first 48 shots of the bench's stream, each with 16 cells, 201.4 Gpts/s in
+      // one launch a step and 211.5 by axis (FP16 222.3 and 238.8); six FP32
+      // shots of 128 to 148 cells a side (0.7 M) 36.3 and 36.8 ms, of 200 to 220
+      // (1.6 M) 75.3 and 74.6.
+      const bool by_axis = form < kCpmlVariants && ends >= kCpmlByAxis;
+      LayerGroup lg{kd, by_axis ? some_axes_group(form) : form, (int)lt.size(), 0, {}, 1, 0};
+      for (const Request *q : of_form) {
         CpmlBatchShot L = q->layer;
         for (int i = 0; i < 6; ++i) {
           L.blk_begin[i] = lg.blocks[i];
-          lg.blocks[i] += cpml_batch_blocks(L, i);
+          lg.blocks[i] += cpml_batch_blocks(L, i, by_axis);
         }
         // about 256 shell receivers per record block, at most 64 blocks a shot
         lg.rec_blocks = std::max(lg.rec_blocks, std::min(64, (L.nsrec + 255) / 256));

@@ -37,14 +37,8 @@ def _submit(srv, made, specs, outs):
             for (grid, storage, steps, npml), (vel, rec, shot), tr in zip(specs, made, outs)]
 
 
-@pytest.mark.parametrize("storages", [(0,), (2, 0, 1)])
-def test_widths_beside_each_other_equal_the_single_grid_path(wave_lib, storages):
+def _served_equals_single(wave_lib, specs):
     import torch
-    specs = [((48 + 5 * i, 61 - 3 * i, 44 + i), storages[i % len(storages)], 30 + 7 * i, w)
-             for i, w in enumerate(WIDTHS + (9, 8))]
-    # axes too short for two unrolled segments, one, two and all three of them
-    specs += [((70, 66, 2 * w + 2), storages[0], 41, w) for w in (8, 16)]
-    specs += [((50, 22, 20), storages[-1], 41, 10), ((41, 43, 40), storages[0], 33, 20)]
     made = [_inputs(grid, npml, i) for i, (grid, _, _, npml) in enumerate(specs)]
     outs = [torch.zeros((sp[2], m[1].shape[0]), device="cuda") for sp, m in zip(specs, made)]
     srv = wave_lib.ShotServer(16 * 10 ** 9, 16)
@@ -63,6 +57,25 @@ def test_widths_beside_each_other_equal_the_single_grid_path(wave_lib, storages)
         s.close()
         assert torch.equal(tr, want), (grid, storage, npml)
         assert float(want.abs().max()) > 0
+
+
+@pytest.mark.parametrize("storage", [0, 2])
+def test_many_line_ends_take_a_launch_per_axis(wave_lib, storage):
+    """1.5 million line ends of a width: one flat shot, or several together."""
+    _served_equals_single(wave_lib, [((850, 849, 24), storage, 60, 8), ((61, 50, 44), storage, 70, 8),
+                                     ((64, 66, 70), storage, 65, 10)])
+    _served_equals_single(wave_lib, [((501 + i, 500 - i, 40), storage, 60 + i, 16) for i in range(3)]
+                          + [((60, 66, 42), storage, 65, 16), ((60, 66, 39), storage, 65, 16)])
+
+
+@pytest.mark.parametrize("storages", [(0,), (2, 0, 1)])
+def test_widths_beside_each_other_equal_the_single_grid_path(wave_lib, storages):
+    specs = [((48 + 5 * i, 61 - 3 * i, 44 + i), storages[i % len(storages)], 30 + 7 * i, w)
+             for i, w in enumerate(WIDTHS + (9, 8))]
+    # axes too short for two unrolled segments, one, two and all three of them
+    specs += [((70, 66, 2 * w + 2), storages[0], 41, w) for w in (8, 16)]
+    specs += [((50, 22, 20), storages[-1], 41, 10), ((41, 43, 40), storages[0], 33, 20)]
+    _served_equals_single(wave_lib, specs)
 
 
 def test_widths_do_not_wait_for_one_another(wave_lib):
