@@ -412,6 +412,16 @@ def cpml_bytes_per_step(shape, npml, esize=4):
     return per_pt * npts + (per_pt * 2 * w + 16 * 2 * npml) * lines
 
 
+def cpml_launches(shape, npml):
+    """Launches of one step with a layer of 8, 10, 16 or 20 cells and two disjoint
+    segments on every axis: the layer's axes together, or one by one from 1.5
+    million line ends; a step's shell receivers ride with the next step's layer."""
+    nx, ny, nz = shape
+    assert npml in (8, 10, 16, 20) and min(shape) >= 2 * (npml + 4)
+    ends = 2 * (nx * ny + ny * nz + nx * nz)
+    return "sweep + 3 axis launches" if ends >= 1500000 else "sweep + 1 layer launch"
+
+
 def cpml_workload(gw, torch, cfg, vel_d, dt, steps, peak_gbs, plain_ms):
     """The same grid and model stepped with the CPML layer at all six faces
     (npml 8 and 16 with FP32 fields, npml 16 with FP16 fields; R = 1e-3,
@@ -447,7 +457,7 @@ def cpml_workload(gw, torch, cfg, vel_d, dt, steps, peak_gbs, plain_ms):
             "roofline": {"bound": "hbm", "achieved": ach, "peak": peak_gbs,
                          "unit": "GB/s", "frac": ach / peak_gbs,
                          "algorithmic_bytes_per_step": b,
-                         "launches_per_step": "sweep + 3 axis kernels + shell receivers"}}
+                         "launches_per_step": cpml_launches((nx, ny, nz), npml)}}
     return out
 
 

@@ -17,11 +17,12 @@
 // afterwards every line along each axis is walked through its two end segments
 // of w cells (one segment of the whole line when the two would overlap), which
 // updates psi_a and zeta_a from u^n (which the sweep does not overwrite) and
-// adds the axis term to u^{n+1}. Corner points are updated by
-// each axis in turn with no race: where every axis holds two disjoint segments
-// of a width they are unrolled for, by one launch over boxes that own their lines whole
-// and a small second one (cpml_lines_kernel); otherwise by axis passes one
-// after another. Receivers within w of a face are then re-recorded.
+// adds the axis term to u^{n+1}. Corner points are updated by each axis in turn
+// with no race. Where every axis holds two disjoint segments of a width they are
+// unrolled for, one launch takes boxes that own their lines whole
+// (cpml_lines_kernel), or one launch per axis where that is faster (kCpmlByAxis,
+// kCpmlByAxisBeside); otherwise axis passes run one after another. Receivers
+// within w of a face are then re-recorded.
 #pragma once
 
 #include <algorithm>
@@ -81,8 +82,14 @@ inline void cpml_axis_coefs(CpmlGeom &g, int ax, double h) {
   }
 }
 
-// Widest layer of the unrolled line ends, and the widths they are built for
-// (each unrolls 6 segments); other layers take the line walks.
+// Widest layer of the unrolled line ends, and the widths they are built for;
+// other layers take the line walks. Each width adds 6 unrolled segments to every
+// kernel of the layer, so the set is small: the widths of the bench and the tests
+// (8, 16) and two common ones beside them (10, 20). Whole steps in us as boxes
+// and as line walks, FP32 and FP16 fields: 150 x 141 x 133 with 8 cells 24 and
+// 44, 25 and 66; with 20 39 and 68, 43 and 106 (12, walks only: 53, 80); 320 x
+// 256 x 192 with 8 68 and 100, 65 and 130; with 20 108 and 143, 102 and 208 (12:
+// 114, 156).
 constexpr int kCpmlMaxCap = 20;
 constexpr int kCpmlVariants = 4;
 
@@ -542,9 +549,10 @@ __global__ void __launch_bounds__(128)
 // line (u^n, psi and zeta; then C and u^{n+1}), on large ones the traffic of
 // lines that every array is read along. Against one launch per axis (line
 // walks at 10 cells, unrolled at 16), with the sweep of that time, a whole step
-// took 31 us instead of 56 at 150 x 141 x 133 with 10 cells (25 now), 102 instead of 104 at 320 x 256 x 192 in
-// FP16 and 291 instead of 296 at 512 x 512 x 256 with 16; the gradient through
-// autograd at 160 x 144 x 128 x 100 steps 18.0 ms instead of 20.0. CTAs of 256
+// took 31 us instead of 56 at 150 x 141 x 133 with 10 cells (25 now), 102 instead
+// of 103 at 320 x 256 x 192 in FP16 (82 now) and 296 instead of 297 at 512 x 512 x
+// 256 with 16 (288 now); the gradient through autograd at 160 x 144 x 128 x 100
+// steps 18.2 ms instead of 20.0 (15.6 now). CTAs of 256
 // threads without clusters took 7 % longer at 320 x 256 x 192, 4 CTAs an SM
 // (128 registers) 2 %, a second launch for the corners' z lines instead of the
 // third phase 4 %, L2 prefetches of C and u^{n+1} 10 %.
@@ -552,7 +560,8 @@ constexpr int kCpmlThreads = 128;
 constexpr int kCpmlCluster = 4;
 constexpr int kCpmlLines = kCpmlThreads * kCpmlCluster;  // lines of a cluster
 
-// CTAs per SM the line kernels are compiled for (168 registers a thread up to 16 cells, 255 beyond).
+// CTAs per SM the line kernels are compiled for (168 registers a thread up to 16
+// cells, 255 beyond; the server's 16-cell forms for 16-bit fields spill 208 bytes).
 constexpr int cpml_ctas(int npml) { return npml > 16 ? 2 : 3; }
 
 // Profile values by axis, face and depth from the face.
@@ -939,7 +948,7 @@ struct CpmlPass {
 // The shell receivers' row of the step before this pass's: u^n is that step's
 // field with the layer's terms, and nothing writes it during this step, so the
 // row rides in blocks beside the lines instead of in a launch of its own after
-// them (3 us a step; the last step's row is recorded at the call's end).
+// them (2 us a step; the last step's row is recorded at the call's end).
 constexpr int kCpmlRecClusters = 8;
 
 template <class T>
