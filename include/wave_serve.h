@@ -88,7 +88,10 @@ typedef struct {
  *   hbm_budget_bytes  device bytes the resident shots may hold (> 0)
  *   max_slots         most shots resident at once (1 .. 4096)
  *   stream            cudaStream_t for all the server's work; NULL: the
- *                     server creates its own non-blocking stream
+ *                     server creates its own non-blocking stream. A
+ *                     batch with layers of several widths or storage types
+ *                     also uses streams of the server's own, joined to this
+ *                     one around each step
  * The current device at this call is the server's device.
  */
 int serve_create(size_t hbm_budget_bytes, int max_slots, void *stream,
