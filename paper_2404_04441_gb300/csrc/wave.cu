@@ -267,7 +267,6 @@ struct KeptWork {
   int contexts = 0;             // wave_ctx alive there
   void *p = nullptr;
   size_t cap = 0;
-  size_t memory = 0;  // of the device
   bool pooled = false;  // a call has been of a size for the pool
   cudaMemPool_t pool = nullptr;
 };
@@ -313,8 +312,7 @@ bool enter_context(unsigned long long home) {
   KeptWork *w = work_of(home);
   for (int i = 0; i < kWorkContexts && !w; ++i)
     if (g_work[i].contexts == 0) w = &g_work[i];
-  size_t avail = 0;
-  if (!w || (w->memory == 0 && cudaMemGetInfo(&avail, &w->memory) != cudaSuccess)) return false;
+  if (!w) return false;
   w->home = home;
   w->contexts++;
   return true;
@@ -329,8 +327,17 @@ void leave_context(unsigned long long home) {
   *w = KeptWork{};
 }
 
+// Memory of the current device (g_work_mu held), asked for once (0.2 ms).
+size_t device_memory_locked(int device) {
+  static size_t known[kWorkContexts] = {};
+  size_t avail = 0, all = 0;
+  size_t &m = device >= 0 && device < kWorkContexts ? known[device] : all;
+  if (m == 0 && cudaMemGetInfo(&avail, &m) != cudaSuccess) m = 0;
+  return m;
+}
+
 // The entry's pool (g_work_mu held), nullptr if there can be none.
-cudaMemPool_t pool_locked(KeptWork &w, int device) {
+cudaMemPool_t pool_locked(KeptWork &w, int device, size_t memory) {
   if (w.pool) return w.pool;
   cudaMemPoolProps props{};
   props.allocType = cudaMemAllocationTypePinned;
@@ -341,7 +348,7 @@ cudaMemPool_t pool_locked(KeptWork &w, int device) {
     cudaGetLastError();
     return nullptr;
   }
-  cuuint64_t keep = w.memory / 16;
+  cuuint64_t keep = memory / 16;
   cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
   return w.pool = pool;
 }
@@ -1569,7 +1576,7 @@ struct Workspace {
   const wave_ctx *c;
   void *block = nullptr;
   size_t cap = 0, bytes = 0;
-  bool keep = false, pooled = false;
+  bool keep = false, small = false, pooled = false;
   std::vector<std::pair<void **, size_t>> asked;
 
   explicit Workspace(const wave_ctx *ctx) : c(ctx) {}
@@ -1583,7 +1590,7 @@ struct Workspace {
     if (keep) {
       std::lock_guard<std::mutex> lock(g_work_mu);
       KeptWork *w = c->counted ? work_of(c->home) : nullptr;
-      if (w && !w->p && cap <= w->memory / 256) {
+      if (w && !w->p && small) {
         w->p = block;
         w->cap = cap;
         return;
@@ -1601,15 +1608,16 @@ struct Workspace {
     if (c->counted) {
       std::lock_guard<std::mutex> lock(g_work_mu);
       KeptWork &w = *work_of(c->home);
-      if (bytes <= w.memory / 256) {
+      const size_t memory = device_memory_locked(c->device);
+      if ((small = bytes <= memory / 256)) {
         if (w.cap >= bytes) {
           block = std::exchange(w.p, nullptr);
           cap = std::exchange(w.cap, 0);
         } else {
           drop_locked(w);  // too small: this call's block is kept instead
         }
-      } else if (bytes <= w.memory / 16) {
-        if (w.pooled) pool = pool_locked(w, c->device);
+      } else if (bytes <= memory / 16) {
+        if (w.pooled) pool = pool_locked(w, c->device, memory);
         w.pooled = true;
       }
     }
